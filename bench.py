@@ -148,7 +148,7 @@ def pass_bytes(plan_geom):
     src = g["nsrc"] * nc * B ** 3 * 4
     dst = g["ndst"] * nc * B ** 3 * 4
     return {"x_fwd_gather_r2c": src + X1, "y_fwd": X1 + X2, "z_fwd_mul_inv": X2 + Kh + X3, "y_inv": X3 + X4,
-            "x_inv_c2r_scatter": X4 + dst}
+            "yz_conv": X1 + Kh + X4, "x_inv_c2r_scatter": X4 + dst}
 
 
 def geometry(src_c, dst_c, ncomp):
@@ -175,10 +175,10 @@ def pass_flops(plan_geom):
 
     def c(n):
         return 5.0 * n * math.log2(n)
+    y_fwd, y_inv = nc * Es[2] * KX * c(N[1]), nc * Et[2] * KX * c(N[1])
+    z = nc * N[1] * KX * (2 * c(N[2]) + 2 * N[2])
     return {"x_fwd_gather_r2c": nc * Es[2] * Es[1] * c(N[0]) / 2,
-            "y_fwd": nc * Es[2] * KX * c(N[1]),
-            "z_fwd_mul_inv": nc * N[1] * KX * (2 * c(N[2]) + 2 * N[2]),
-            "y_inv": nc * Et[2] * KX * c(N[1]),
+            "y_fwd": y_fwd, "z_fwd_mul_inv": z, "y_inv": y_inv, "yz_conv": y_fwd + z + y_inv,
             "x_inv_c2r_scatter": nc * Et[2] * Et[1] * c(N[0]) / 2}
 
 
@@ -388,15 +388,17 @@ def bench_gpu(args):
     value = job_rate(pts_per_step, args.steps, ws, dev_ms / 1e3)
     e2e_value = job_rate(pts_per_step, e2e_steps, ws, e2e_s)
     # roofline of the dominant kernel, on the algorithmic bytes of the path: 8 B per target
-    # point (4 B FP32 source in, 4 B result out); one launch of a pass is one component
-    g1 = geometry(src_c, dst_c, 1)
+    # point (4 B FP32 source in, 4 B result out); one launch of a pass is all three components
+    # in the three-pass form, one component in the five-pass form
+    per = 3 if "yz_conv" in kt else 1
+    g1 = geometry(src_c, dst_c, per)
     pb = pass_bytes(g1)
     pf = pass_flops(g1)
     dom = max(kt, key=lambda k: kt[k][1])
     launches, tot_ms = kt[dom]
     per_launch_ms = tot_ms / launches
     hbm, src_kind = peaks()
-    alg_bytes = 8 * len(dst_c) * B ** 3            # one component
+    alg_bytes = 8 * per * len(dst_c) * B ** 3
     achieved = alg_bytes / (per_launch_ms / 1e3) / 1e9
     if dom not in pb:      # the autotuner chose the split solve: no per-pass workspace or flop model
         pb[dom], pf[dom] = 0, 0.0
@@ -404,8 +406,8 @@ def bench_gpu(args):
     roof = {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
             "frac": round(achieved / hbm, 4), "traffic": None,
             "algorithmic_bytes_per_launch": alg_bytes, "mean_launch_ms": round(per_launch_ms, 5),
-            "bytes_rule": "8 B per target point and component (FP32 source read + result write), one component "
-                          "per launch",
+            "bytes_rule": "8 B per target point and component (FP32 source read + result write), %d component(s) "
+                          "per launch" % per,
             "step": {"achieved": round(step_gbs, 1), "frac": round(step_gbs / hbm, 4),
                      "rule": "8 B per target point and component over the whole timed step"},
             "pass_workspace": {"bytes_per_launch": pb[dom],
@@ -414,8 +416,7 @@ def bench_gpu(args):
                                "rule": "the pass's own input and output arrays (complex FP32 workspaces, "
                                        "kernel spectrum): bytes of this algorithm, not of the path"},
             "traffic_note": "DRAM bytes per launch (ncu) are in profiles/poisson_ring128_ncu.md",
-            "launch_timing": "CUDA events around each launch (one pass of one component) in K profiled steps "
-                             "after the timed ones; profiling runs the components one after another",
+            "launch_timing": "CUDA events around each launch (one pass) in K profiled steps after the timed ones",
             "peak_source": src_kind + " (MEASURED_PEAKS.json hbm_gbs)" if src_kind == "measured" else src_kind}
     comp_tf = pf[dom] / (per_launch_ms / 1e3) / 1e12
     compute = {"bound": "fp32", "kernel": dom, "achieved": round(comp_tf, 2), "peak": peaks_tf["fp32_fma"],
@@ -442,7 +443,8 @@ def bench_gpu(args):
     cfg.update({"method": {"chosen": ["whole-box FFT convolution", "block-sparse split solve"][chosen],
                            "autotune_ms": {"whole_box": round(auto_wb, 4), "split": round(auto_split, 4)},
                            "rule": "lgf_conv_plan method 2: both planned, one timed execution each, the faster kept"},
-                "fft_grid": geom["N"], "execution": "one stream per component, launch sequence replayed as a CUDA graph",
+                "fft_grid": geom["N"], "execution": "%s, launch sequence replayed as a CUDA graph" %
+                ("three passes, all components per launch" if per == 3 else "one stream per component"),
                 "plain_ms": round(plain_ms, 4), "batched_over_plain": round(plain_ms / (dev_ms / args.steps), 3),
                 "plain": "one component per solve, three solves one after another on one stream, no graph",
                 "l2": "256 MiB buffer rewritten between timed steps (outside the events)",

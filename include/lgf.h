@@ -152,7 +152,10 @@ void lgf_table_destroy(lgf_table *t);
  * the smallest of 16, 32, 64, 96, 128, 192, 256, 288, 384, 432, 512, 768, 1024 that is
  * >= max(2 m + 2, 2 E), m the largest |target - source| offset and E the
  * source extent (points); at most 1024 (FP32) or 512 (FP64), else
- * LGF_ERR_ARG.  The table must outlive the
+ * LGF_ERR_ARG.  The table has to reach half that length on every axis.  FP32
+ * solves whose axes fit 512 points run in three passes on lengths of their own,
+ * multiples of 16 or 32 with the same exact embedding (where that is the faster
+ * form).  The table must outlive the
  * plan.  Synchronises `stream`.  opts may be NULL (defaults).
  * ------------------------------------------------------------------------- */
 lgf_status lgf_conv_plan(const lgf_table *t, const lgf_solve_desc *solves, int n_solves,
@@ -369,9 +372,9 @@ const char *lgf_last_error(void);
 /* Library version string. */
 const char *lgf_version(void);
 
-/* The FFT length a Poisson plan takes for an axis that needs at least `need`
- * points (the size rule of lgf_conv_plan): the smallest supported length
- * >= need, 0 if none.  Host only; no CUDA call. */
+/* The FFT length by which a Poisson plan is sized for an axis that needs at least
+ * `need` points (the size rule of lgf_conv_plan, for table sizes): the smallest
+ * supported length >= need, 0 if none.  Host only; no CUDA call. */
 int lgf_fft_length(int need);
 
 #ifdef __cplusplus

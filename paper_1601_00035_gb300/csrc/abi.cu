@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "plan.hpp"
+#include "plane.hpp"
 #include "poisson_passes.hpp"
 
 namespace lgf {
@@ -89,16 +90,21 @@ void free_plan(lgf_plan *p)
         cudaFree(ps.d_dst2src);
         cudaFree(ps.d_stage_src);
         cudaFree(ps.d_stage_dst);
+        cudaFree(ps.d_twf);
+        cudaFree(ps.d_twi);
     }
     for (auto &sp : p->spectra) cudaFree(sp.d_Kh);
+    for (auto &sp : p->spectra) cudaFree(sp.d_Kt);
     cudaFree(p->d_wsA);
     cudaFree(p->d_wsB);
     cudaFree(p->d_wsA64);
     cudaFree(p->d_wsB64);
     for (auto &sp : p->spectra) cudaFree(sp.d_Kh64);
     for (auto e : p->unit_mark) cudaEventDestroy(e);
-    for (auto w : p->lane_wsA) cudaFree(w);
-    for (auto w : p->lane_wsB) cudaFree(w);
+    if (!p->merged) {  // (merged: slices of d_wsA, d_wsB)
+        for (auto w : p->lane_wsA) cudaFree(w);
+        for (auto w : p->lane_wsB) cudaFree(w);
+    }
     for (auto st : p->lanes) cudaStreamDestroy(st);
     for (auto e : p->lane_done) cudaEventDestroy(e);
     if (p->fork) cudaEventDestroy(p->fork);
@@ -403,11 +409,14 @@ static lgf_status plan_grouped(lgf_plan *p, cudaStream_t s)
     std::vector<double> cost;
     for (int i = 0; i < nu; i++) {
         const Geom &g0 = p->solves[p->units[i].solve].g;
-        const std::vector<int> key = {g0.N[0], g0.N[1], g0.N[2]};
+        const PoissonSolve &q0 = p->solves[p->units[i].solve];
+        const std::vector<int> key = q0.plane ? std::vector<int>{1, q0.pg.Mx, q0.pg.Dy, q0.pg.My, q0.pg.Mz}
+                                              : std::vector<int>{0, g0.N[0], g0.N[1], g0.N[2]};
         auto it = by_grid.find(key);
         if (it == by_grid.end()) {
             it = by_grid.emplace(key, (int)p->groups.size()).first;
             p->groups.emplace_back();
+            p->groups.back().plane = q0.plane;
             cost.push_back(0.0);
         }
         p->groups[it->second].units.push_back(i);
@@ -416,35 +425,57 @@ static lgf_status plan_grouped(lgf_plan *p, cudaStream_t s)
     const int ng = (int)p->groups.size();
     for (int gi = 0; gi < ng; gi++) {
         lgf_plan::Group &gr = p->groups[gi];
-        for (int pass = 0; pass < 5; pass++) {
+        const PoissonSolve &q0 = p->solves[p->units[gr.units[0]].solve];
+        const int npass = gr.plane ? 3 : 5;
+        gr.pass.resize(npass);
+        for (int pass = 0; pass < npass; pass++) {
             std::vector<GroupTask<float>> tasks;
+            std::vector<PlaneTask> ptasks;
             std::vector<int> cta;
+            lgf_plan::GroupLaunch &L = gr.pass[pass];
+            L = {pass, 0, 0, 0, 0, 0, nullptr, nullptr};
             for (int i : gr.units) {
                 const auto &u = p->units[i];
-                Geom g = p->solves[u.solve].g;
-                g.c0 = u.c0;
-                g.nc = 1;
-                const int nt = poisson_tiles(pass, g);
-                LGF_CHECK_ARG(nt >= 0, "grouped plan: unsupported FFT length %d", g.N[pass_axis(pass)]);
-                GroupTask<float> t;
-                t.g = g;
-                t.wa = p->unit_wa[i];
-                t.wb = p->unit_wb[i];
-                t.solve = u.solve;
-                t.first = (int)cta.size();
-                cta.insert(cta.end(), nt, (int)tasks.size());
-                tasks.push_back(t);
+                const PoissonSolve &q = p->solves[u.solve];
+                int nt;
+                if (gr.plane) {
+                    PlaneTask t{q.pg, p->unit_wa[i], p->unit_wb[i], u.solve, (int)cta.size()};
+                    t.g.c0 = u.c0;
+                    t.g.nc = 1;
+                    nt = plane_tiles(pass, t.g);
+                    L.smem = std::max(L.smem, plane_smem(pass, t.g));
+                    cta.insert(cta.end(), nt, (int)ptasks.size());
+                    ptasks.push_back(t);
+                } else {
+                    GroupTask<float> t;
+                    t.g = q.g;
+                    t.g.c0 = u.c0;
+                    t.g.nc = 1;
+                    nt = poisson_tiles(pass, t.g);
+                    LGF_CHECK_ARG(nt >= 0, "grouped plan: unsupported FFT length %d", t.g.N[pass_axis(pass)]);
+                    t.wa = p->unit_wa[i];
+                    t.wb = p->unit_wb[i];
+                    t.solve = u.solve;
+                    t.first = (int)cta.size();
+                    cta.insert(cta.end(), nt, (int)tasks.size());
+                    tasks.push_back(t);
+                }
             }
-            lgf_plan::GroupLaunch &L = gr.pass[pass];
-            L.pass = pass;
-            L.n = p->solves[p->units[gr.units[0]].solve].g.N[pass_axis(pass)];
+            L.threads = gr.plane ? q0.pg.ntz : 0;
+            L.Dy = gr.plane ? q0.pg.Dy : 0;
+            L.n = gr.plane ? (pass == 1 ? q0.pg.Mz : q0.pg.Mx) : q0.g.N[pass_axis(pass)];
             L.ncta = (int)cta.size();
-            L.d_tasks = nullptr;
-            L.d_cta = nullptr;
-            GroupTask<float> *dt = nullptr;
-            LGF_TRY(dalloc(&dt, tasks.size(), p->bytes));
-            L.d_tasks = dt;
-            LGF_TRY(upload(dt, tasks, s));
+            if (gr.plane) {
+                PlaneTask *dt = nullptr;
+                LGF_TRY(dalloc(&dt, ptasks.size(), p->bytes));
+                L.d_tasks = dt;
+                LGF_TRY(upload(dt, ptasks, s));
+            } else {
+                GroupTask<float> *dt = nullptr;
+                LGF_TRY(dalloc(&dt, tasks.size(), p->bytes));
+                L.d_tasks = dt;
+                LGF_TRY(upload(dt, tasks, s));
+            }
             LGF_TRY(dalloc(&L.d_cta, cta.size(), p->bytes));
             LGF_TRY(upload(L.d_cta, cta, s));
         }
@@ -473,8 +504,11 @@ static lgf_status plan_grouped(lgf_plan *p, cudaStream_t s)
 static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_desc *solves, int n_solves, cudaStream_t s)
 {
     LGF_TRY(poisson_prepare());
+    if (p->precision == 0) LGF_TRY(plane_prepare());
     std::map<std::vector<int>, int> spec_index;
     size_t maxA = 0, maxB = 0;
+    int n_units = 0;
+    for (int i = 0; i < n_solves; i++) n_units += solves[i].ncomp;
     for (int i = 0; i < n_solves; i++) {
         const lgf_solve_desc &d = solves[i];
         LGF_CHECK_ARG(d.B == 8 || d.B == 16 || d.B == 32, "solve %d: B=%d not in {8,16,32}", i, d.B);
@@ -500,6 +534,7 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
         ps.scale = d.scale;
         ps.src_coords.assign(d.src_blocks, d.src_blocks + 3 * d.n_src);
         ps.dst_coords.assign(d.dst_blocks, d.dst_blocks + 3 * d.n_dst);
+        long mabs[3];  // largest |target - source| offset per axis
         int smin[3], smax[3], tmin[3], tmax[3];
         for (int a = 0; a < 3; a++) {
             smin[a] = tmin[a] = 1 << 30;
@@ -525,6 +560,7 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
             const long lo = (long)g.T0[a] - (long)(g.S0[a] + g.Es[a] - 1);
             const long hi = (long)(g.T0[a] + g.Et[a] - 1) - (long)g.S0[a];
             const long maxabs = std::max(std::labs(lo), std::labs(hi));
+            mabs[a] = maxabs;
             // exact embedding: N >= 2 maxabs + 2 (no two offsets share a wrapped
             // index); N >= 2 Es keeps every source sample in the lower half of
             // the line, which the forward transforms take as their zero pattern
@@ -534,6 +570,8 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
                           maxabs, a);
             g.N[a] = n;
         }
+        ps.plane = p->precision == 0 && plane_pick(g, mabs, n_units, ps.pg);
+        if (ps.plane) LGF_TRY(plane_tables(ps.pg));
         g.KX = g.N[0] / 2 + 1;
         g.mul = (float)(d.scale * d.dx * d.dx / ((double)g.N[0] * g.N[1] * g.N[2]));
         // lookups
@@ -573,12 +611,53 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
         q.g.src_lut = q.d_src_lut;
         q.g.dst_lut = q.d_dst_lut;
         const size_t KX = g.KX, nc = d.ncomp;
-        q.elemsA = std::max(nc * g.Es[2] * g.Es[1] * KX, nc * g.Et[2] * (size_t)g.N[1] * KX);
-        q.elemsB = std::max(nc * g.Es[2] * (size_t)g.N[1] * KX, nc * g.Et[2] * g.Et[1] * KX);
+        if (q.plane) {
+            PlaneGeom &pg = q.pg;
+            pg.src_lut = q.d_src_lut;
+            pg.dst_lut = q.d_dst_lut;
+            pg.mul = (float)(d.scale * d.dx * d.dx / ((double)pg.Mx * pg.Dy * pg.My * 2 * pg.Mz));
+            const double tau = 6.28318530717958647692, Ny = pg.Dy * pg.My;
+            std::vector<float2> wf, wi;  // w_Ny^(r n) of the source rows, conj w_Ny^(r p) of the target rows
+            for (int r = 0; r < pg.Dy; r++) {
+                for (int n = 0; n < g.Es[1]; n++) {
+                    const double t = -tau * std::fmod((double)r * n, Ny) / Ny;
+                    wf.push_back(make_float2((float)std::cos(t), (float)std::sin(t)));
+                }
+                for (int n = 0; n < g.Et[1]; n++) {
+                    const double t = tau * std::fmod((double)r * (n + pg.d0[1]), Ny) / Ny;
+                    wi.push_back(make_float2((float)std::cos(t), (float)std::sin(t)));
+                }
+            }
+            LGF_TRY(dalloc(&q.d_twf, wf.size(), p->bytes));
+            LGF_TRY(dalloc(&q.d_twi, wi.size(), p->bytes));
+            LGF_TRY(upload(q.d_twf, wf, s));
+            LGF_TRY(upload(q.d_twi, wi, s));
+            pg.twf = q.d_twf;
+            pg.twi = q.d_twi;
+            q.elemsA = nc * plane_elems_a(pg);
+            q.elemsB = nc * plane_elems_b(pg);
+        } else {
+            q.elemsA = std::max(nc * g.Es[2] * g.Es[1] * KX, nc * g.Et[2] * (size_t)g.N[1] * KX);
+            q.elemsB = std::max(nc * g.Es[2] * (size_t)g.N[1] * KX, nc * g.Et[2] * g.Et[1] * KX);
+        }
         maxA = std::max(maxA, q.elemsA);
         maxB = std::max(maxB, q.elemsB);
-        std::vector<int> key = {g.N[0], g.N[1], g.N[2]};
+        // the table has to reach half the padded lengths of the library's size rule
+        // (lgf_fft_length), whichever form runs
+        LGF_TRY(check_table_reach(t->K, g.N));
+        std::vector<int> key = {0, g.N[0], g.N[1], g.N[2]};
+        // three-pass form: samples beyond Kn are zero (no valid output uses them), so that the
+        // spectrum does not depend on how far beyond its need the table reaches
+        const int Kn = std::max(g.N[0], std::max(g.N[1], g.N[2])) / 2 - 1;
+        if (q.plane) key = {1, q.pg.Mx, q.pg.Dy, q.pg.My, q.pg.Mz, Kn};
         auto it = spec_index.find(key);
+        if (it == spec_index.end() && q.plane) {
+            p->spectra.emplace_back();
+            Spectrum &spr = p->spectra.back();
+            LGF_TRY(dalloc(&spr.d_Kt, plane_spectrum_size(q.pg), p->bytes));
+            LGF_TRY(plane_spectrum(t->d_vals, Kn, q.pg, spr.d_Kt, s));
+            it = spec_index.emplace(key, (int)p->spectra.size() - 1).first;
+        }
         if (it == spec_index.end()) {
             Spectrum sp;
             sp.N[0] = g.N[0];
@@ -596,6 +675,7 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
     }
     for (auto &q : p->solves) {
         q.g.Kh = p->spectra[q.spec].d_Kh;
+        q.pg.Kt = p->spectra[q.spec].d_Kt;
         q.g.Kh64 = p->spectra[q.spec].d_Kh64;
         q.g.mul64 = q.scale * q.dx * q.dx / ((double)q.g.N[0] * q.g.N[1] * q.g.N[2]);
     }
@@ -608,12 +688,15 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
         LGF_TRY(dalloc(&p->d_wsB64, maxB, p->bytes));
         return LGF_OK;
     }
-    if (n_solves == 1 && p->solves[0].g.ncomp == 1) {
+    // one solve in the three-pass form: all components in one launch per pass (device buffers); the
+    // per-component units below, on slices of the same workspaces, serve host buffers
+    p->merged = n_solves == 1 && p->solves[0].plane;
+    if (p->merged || (n_solves == 1 && p->solves[0].g.ncomp == 1)) {
         LGF_TRY(dalloc(&p->d_wsA, maxA, p->bytes));
         LGF_TRY(dalloc(&p->d_wsB, maxB, p->bytes));
         p->wsA = maxA;
         p->wsB = maxB;
-        return LGF_OK;
+        if (p->solves[0].g.ncomp == 1) return LGF_OK;
     }
     // Several independent units, one per (solve, component): each runs the five
     // passes on its own worker stream (up to 4), so the passes of different
@@ -654,6 +737,11 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
     for (int k = 0; k < nl; k++) {
         LGF_CUDA_TRY(cudaStreamCreateWithFlags(&p->lanes[k], cudaStreamNonBlocking));
         LGF_CUDA_TRY(cudaEventCreateWithFlags(&p->lane_done[k], cudaEventDisableTiming));
+        if (p->merged) {
+            p->lane_wsA[k] = p->d_wsA + k * la[k];
+            p->lane_wsB[k] = p->d_wsB + k * lb[k];
+            continue;
+        }
         LGF_TRY(dalloc(&p->lane_wsA[k], la[k], p->bytes));
         LGF_TRY(dalloc(&p->lane_wsB[k], lb[k], p->bytes));
     }
@@ -1000,16 +1088,25 @@ static lgf_status run_poisson(lgf_plan *p, const float *const *src, float *const
         const PoissonSolve &q = p->solves[u.solve];
         if (wait) LGF_CUDA_TRY(cudaStreamWaitEvent(st, wait, 0));
         if (host) LGF_TRY(copy_slice((float *)src[u.solve], host->src[u.solve], q, q.nsrc, u.c0, u.nc, true, st));
-        LGF_TRY(poisson_launch(unit_geom(u), src[u.solve], dst[u.solve], wa, wb, st, pr, mark, mark ? 0 : -1));
+        if (q.plane) {
+            PlaneGeom pg = q.pg;
+            pg.c0 = u.c0;
+            pg.nc = u.nc;
+            LGF_TRY(plane_launch(pg, src[u.solve], dst[u.solve], wa, wb, st, pr, mark, mark ? 0 : -1));
+        } else {
+            LGF_TRY(poisson_launch(unit_geom(u), src[u.solve], dst[u.solve], wa, wb, st, pr, mark, mark ? 0 : -1));
+        }
         if (host) LGF_TRY(copy_slice(dst[u.solve], host->dst[u.solve], q, q.ndst, u.c0, u.nc, false, st));
         return LGF_OK;
     };
     if (p->grouped) {
         SolvePtrs<float> ptrs;
+        PlanePtrs pptrs;
         for (size_t i = 0; i < p->solves.size(); i++) {
-            ptrs.src[i] = src[i];
-            ptrs.dst[i] = dst[i];
+            ptrs.src[i] = pptrs.src[i] = src[i];
+            ptrs.dst[i] = pptrs.dst[i] = dst[i];
         }
+        static const char *pnames[3] = {"x_fwd_gather_r2c", "yz_conv", "x_inv_c2r_scatter"};
         static const char *names[5] = {"x_fwd_gather_r2c", "y_fwd", "z_fwd_mul_inv", "y_inv", "x_inv_c2r_scatter"};
         // one group on stream st: its units' copies in, five grouped launches, copies out
         auto run_group = [&](const lgf_plan::Group &gr, cudaStream_t st, Profiler *pr) -> lgf_status {
@@ -1021,9 +1118,13 @@ static lgf_status run_poisson(lgf_plan *p, const float *const *src, float *const
                 }
             for (const auto &gl : gr.pass) {
                 if (pr) pr->begin(st);
-                LGF_TRY(poisson_launch_grouped(gl.pass, gl.n, (const GroupTask<float> *)gl.d_tasks, gl.d_cta, gl.ncta,
-                                               ptrs, st));
-                if (pr) pr->end(names[gl.pass], st);
+                if (gr.plane)
+                    LGF_TRY(plane_pass_grouped(gl.pass, gl.n, gl.smem, gl.threads, gl.Dy, (const PlaneTask *)gl.d_tasks, gl.d_cta, gl.ncta,
+                                               pptrs, st));
+                else
+                    LGF_TRY(poisson_launch_grouped(gl.pass, gl.n, (const GroupTask<float> *)gl.d_tasks, gl.d_cta,
+                                                   gl.ncta, ptrs, st));
+                if (pr) pr->end(gr.plane ? pnames[gl.pass] : names[gl.pass], st);
             }
             if (host)
                 for (int i : gr.units) {
@@ -1046,7 +1147,7 @@ static lgf_status run_poisson(lgf_plan *p, const float *const *src, float *const
         }
         return LGF_OK;
     }
-    if (p->lanes.empty()) {
+    if (p->lanes.empty() || (p->merged && !host)) {
         for (size_t i = 0; i < p->solves.size(); i++)
             LGF_TRY(run_unit({(int)i, 0, p->solves[i].g.ncomp, 0, 0, 0}, p->d_wsA, p->d_wsB, s, prof));
         return LGF_OK;

@@ -29,8 +29,35 @@ struct Geom {
     int KX;              // Nx/2 + 1
 };
 
+// In-place two-factor lengths M = R1 * R2: multiples of 16 up to 256.
+constexpr int kPlaneMax = 256;
+constexpr int kPlaneMaxD = 4;  // residues of ky (cluster size of the yz pass)
+
+// Geometry of one solve in the three-pass form (POD, a kernel parameter).
+// Axis order 0 = x, 1 = y, 2 = z.  Nx = 2 Mx, Ny = Dy * My, Nz = 2 Mz.
+struct PlaneGeom {
+    int B, lB, ncomp;    // block edge, its log2, components per point of the block layout
+    int c0, nc;          // components c0 .. c0 + nc - 1 in this launch
+    int Es[3], Et[3];    // source / target box extents
+    int d0[3];           // target origin - source origin
+    int nbS[3], nbT[3];  // the boxes in blocks
+    int Mx, KX;          // KX = Mx + 1 kept x frequencies
+    int Dy, My, Ry1, Ry2;
+    int Mz, ntz;         // ntz: threads per block of the yz pass
+    float mul;           // scale * dx^2 / (Mx Ny Nz)
+    const int *src_lut, *dst_lut;
+    const float *Kt;         // kernel spectrum [kx][r][Mz + 1][My] in the planes' order
+    const float2 *twf;       // [Dy][Es_y]  w_Ny^(r n): fold of the source rows
+    const float2 *twi;       // [Dy][Et_y]  conj w_Ny^(r p), p the target's position
+    const float2 *st[3];     // stage twiddles of Mx, My, Mz: [R2][R1] w_M^(b q)
+    const float2 *w2[3];     // w_2M^n, n <= M, of Mx (My unused) and Mz
+};
+
 struct PoissonSolve {
     Geom g;
+    bool plane = false;  // executed in the three-pass form (plane.hpp), with the geometry pg
+    PlaneGeom pg;
+    float2 *d_twf = nullptr, *d_twi = nullptr;
     int nsrc, ndst;
     double dx, scale;
     std::vector<int32_t> src_coords, dst_coords;  // host copies
@@ -46,6 +73,7 @@ struct Spectrum {
     int N[3];
     float *d_Kh = nullptr;
     double *d_Kh64 = nullptr;  // FP64 plans
+    float *d_Kt = nullptr;     // three-pass form (plane.hpp); d_Kh is then not built
 };
 
 // Optional per-kernel event timing (lgf_plan_set_profiling).
@@ -84,6 +112,8 @@ lgf_status poisson_prepare();  // per-device constant tables; call outside strea
 int poisson_pick_n(int need);  // smallest supported FFT length >= need, 0 if none
 
 // spectrum construction (spectrum.cu): FP64 cosine transforms of the table samples
+// K: the table's max_offset; samples beyond it, which no valid output may use, are zero
+lgf_status check_table_reach(int K, const int N[3]);  // LGF_ERR_ARG unless the table reaches every sample
 lgf_status build_spectrum(const double *d_octant, int K, const int N[3], float *d_Kh, double *d_Kh64,
                           cudaStream_t s);
 
@@ -273,6 +303,7 @@ struct lgf_plan {
     lgf::cx<double> *d_wsA64 = nullptr, *d_wsB64 = nullptr;
     // several solves: worker streams ("lanes"), each with its own workspaces;
     // execute forks them off the caller's stream with events and joins back
+    bool merged = false;  // one three-pass solve: device buffers take all components per launch
     std::vector<cudaStream_t> lanes;
     std::vector<cudaEvent_t> lane_done;
     cudaEvent_t fork = nullptr;
@@ -292,13 +323,16 @@ struct lgf_plan {
     std::vector<lgf::cx<float> *> unit_wa, unit_wb;
     struct GroupLaunch {
         int pass, n, ncta;
-        void *d_tasks;  // GroupTask<float>[]
+        size_t smem;    // dynamic shared memory, threads and cluster size of the yz pass (three-pass form)
+        int threads, Dy;
+        void *d_tasks;  // GroupTask<float>[] or PlaneTask[]
         int *d_cta;     // task of every thread block
     };
     struct Group {
         int lane;
+        bool plane;             // three-pass form
         std::vector<int> units;
-        GroupLaunch pass[5];
+        std::vector<GroupLaunch> pass;
     };
     std::vector<Group> groups;
     double *d_acc = nullptr;  // residual accumulators

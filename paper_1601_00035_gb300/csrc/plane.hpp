@@ -1,0 +1,75 @@
+// Three-pass FP32 form of the Poisson solve (kernels in plane_kernels.cuh):
+//   x forward   gather, real transform along x, transposed store
+//   yz          per (kx, residue of ky): transform along y, convolution along z,
+//               inverse along y, all in one shared-memory plane
+//   x inverse   recombination of the ky residues, real inverse along x, scatter
+// against the five passes of poisson.cu (which FP64 plans and boxes beyond the lengths here keep).
+#pragma once
+#include "plan.hpp"
+
+namespace lgf {
+
+struct PlaneTask {  // one unit of a grouped launch
+    PlaneGeom g;
+    cx<float> *wa, *wb;
+    int solve, first;
+};
+constexpr int kPlaneMaxSolves = 128;
+struct PlanePtrs {
+    const float *src[kPlaneMaxSolves];
+    float *dst[kPlaneMaxSolves];
+};
+
+// lengths for a solve (g: boxes and origins set; maxabs: largest |target - source| offset per
+// axis); false where the five-pass form is the one to take
+// units: (solve, component) pairs whose launches share the GPU
+bool plane_pick(const Geom &g, const long maxabs[3], int units, PlaneGeom &out);
+lgf_status plane_prepare();                 // per-device tables and kernel attributes
+lgf_status plane_tables(PlaneGeom &g);      // fills st, w2 from the per-device tables
+lgf_status plane_spectrum(const double *d_octant, int K, const PlaneGeom &g, float *d_Kt, cudaStream_t s);
+inline size_t plane_spectrum_size(const PlaneGeom &g) { return (size_t)g.KX * g.Dy * (g.Mz + 1) * g.My; }
+inline size_t plane_elems_a(const PlaneGeom &g) { return (size_t)g.KX * g.Es[1] * g.Es[2]; }          // per component
+inline size_t plane_elems_b(const PlaneGeom &g) { return (size_t)g.KX * g.Et[1] * g.Et[2]; }
+int plane_tiles(int pass, const PlaneGeom &g);  // thread blocks of one component (pass 0, 1, 2)
+lgf_status plane_pass(int pass, const PlaneGeom &g, const float *src, float *dst, cx<float> *wa, cx<float> *wb,
+                      cudaStream_t s);
+lgf_status plane_pass_grouped(int pass, int M, size_t smem, int threads, int Dy, const PlaneTask *tasks, const int *cta, int ncta,
+                              const PlanePtrs &ptrs, cudaStream_t s);
+size_t plane_smem(int pass, const PlaneGeom &g);
+lgf_status plane_launch(const PlaneGeom &g, const float *src, float *dst, cx<float> *wa, cx<float> *wb, cudaStream_t s,
+                        Profiler *prof = nullptr, cudaEvent_t mark = nullptr, int mark_after = -1);
+
+// per length M (multiple of 16): the launches, instantiated in the plane_*.cu units
+template <int M>
+struct PlaneX {
+    static lgf_status prepare();
+    static lgf_status fwd(const PlaneGeom &g, const float *src, cx<float> *a, cudaStream_t s);
+    static lgf_status inv(const PlaneGeom &g, const cx<float> *b, float *dst, cudaStream_t s);
+    static lgf_status fwd_grp(const PlaneTask *t, const int *cta, int ncta, size_t smem, const PlanePtrs &p, cudaStream_t s);
+    static lgf_status inv_grp(const PlaneTask *t, const int *cta, int ncta, size_t smem, const PlanePtrs &p, cudaStream_t s);
+};
+template <int M>
+struct PlaneYZ {
+    static lgf_status prepare();
+    static lgf_status run(const PlaneGeom &g, const cx<float> *a, cx<float> *b, cudaStream_t s);
+    static lgf_status grp(const PlaneTask *t, const int *cta, int ncta, size_t smem, int threads, int Dy,
+                          cudaStream_t s);
+};
+
+// radices of M = R1 * R2 (R2 even)
+__host__ __device__ constexpr int plane_r2(int M)
+{
+    return M <= 32 ? 4 : M == 48 ? 6 : M <= 128 ? 8 : M == 144 ? 12 : M == 160 ? 10 : M == 192 ? 12 : M == 224 ? 14 : 16;
+}
+__host__ __device__ constexpr int plane_r1(int M) { return M / plane_r2(M); }
+// the z transform's second radix (even), and the threads per SM its registers leave room for
+__host__ __device__ constexpr int plane_z2(int M)
+{
+    return M == 16 ? 4 : (M <= 80 ? 8 : 16);
+}
+__host__ __device__ constexpr int plane_yz_threads(int M) { return M <= 128 ? 1024 : M <= 192 ? 768 : 512; }
+
+#define LGF_PLANE_LENGTHS(X) \
+    X(16) X(32) X(48) X(64) X(80) X(96) X(112) X(128) X(144) X(160) X(176) X(192) X(208) X(224) X(240) X(256)
+
+}  // namespace lgf

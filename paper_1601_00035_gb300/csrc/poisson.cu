@@ -5,6 +5,9 @@
 // The kernel samples G(wrap(j)) are real and even, so their spectrum is real
 // and even and only its octant is stored (built in FP64, spectrum.cu).
 //
+// FP32 solves whose axes fit 512 points run in the three-pass form of plane.hpp where that is
+// faster; this unit holds the general five-pass form (FP64, longer axes, lopsided boxes).
+//
 // Five passes, each a batch of register-resident 1-D FFTs (fft.cuh):
 //   x_fwd : gather source rows from the block list (two real rows packed into
 //           one complex line), R2C along x                 src -> A[c][z][y][kx]

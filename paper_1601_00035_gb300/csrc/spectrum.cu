@@ -77,15 +77,20 @@ __global__ void k_to_f32(const double *__restrict__ in, float *__restrict__ out,
 
 }  // namespace
 
+lgf_status check_table_reach(int K, const int N[3])
+{
+    const int n = std::max(N[0], std::max(N[1], N[2]));
+    if (n / 2 - 1 > K) {
+        set_error("table max_offset %d too small for FFT grid (%d,%d,%d): need %d", K, N[0], N[1], N[2], n / 2 - 1);
+        return LGF_ERR_ARG;
+    }
+    return LGF_OK;
+}
+
 lgf_status build_spectrum(const double *d_octant, int K, const int N[3], float *d_Kh, double *d_Kh64,
                           cudaStream_t s)
 {
     const int hx = N[0] / 2, hy = N[1] / 2, hz = N[2] / 2;
-    if (hx - 1 > K || hy - 1 > K || hz - 1 > K) {
-        set_error("table max_offset %d too small for FFT grid (%d,%d,%d): need %d", K, N[0], N[1], N[2],
-                  (N[0] > N[1] ? (N[0] > N[2] ? N[0] : N[2]) : (N[1] > N[2] ? N[1] : N[2])) / 2 - 1);
-        return LGF_ERR_ARG;
-    }
     const int nx = hx + 1, ny = hy + 1, nz = hz + 1;
     const int64_t total = (int64_t)nx * ny * nz;
     double *a = nullptr, *b = nullptr, *ct = nullptr;
