@@ -20,6 +20,17 @@
 // neighbours) into registers and produces its B outputs with the symmetric
 // taps (g0 v + sum_d g_d (v_{+d} + v_{-d})).  Taps travel as kernel parameters
 // (constant bank), padded with zeros up to the instantiated radius RM.
+//
+// The 128^3 fields of three components (25 MB, kept in L2) are bound by instruction issue and by
+// the launches' ramps, larger ones by HBM (the 256^3 ring's 1251 blocks: y 122 MB in 28 us, z with
+// a combination 183 MB in 37 us).  The y and x launches therefore overlap their predecessor's end
+// (programmatic dependent launch; three applications on 128^3 at R = 7, 9, 15: 122 -> 110 us); the
+// z launch does not (behind the shared-memory passes of a Poisson solve it would start on their
+// shared-memory carveout: the ring's step 1440 against 1428 us).  The y and x passes read by
+// ordinary loads (__ldca): loads through the read-only path may be taken before the wait for the
+// pass that writes their input.  Runs of two or four output blocks per thread block with the window
+// kept in registers, fewer reads from L2, measured the same; rows staged in shared memory for the x
+// pass 40 against 34 us on the ring.
 #include "plan.hpp"
 
 namespace lgf {
@@ -29,6 +40,14 @@ template <int RM>
 struct Taps {
     float g[RM + 1];
 };
+
+// the z pass reads what complete launches wrote, the others their predecessor's output
+template <int AXIS, typename V>
+__device__ __forceinline__ V if_load(const V *p)
+{
+    if constexpr (AXIS == 2) return __ldg(p);
+    else return __ldca(p);
+}
 
 // AXIS 2: z pass (thread per (x, y)), AXIS 1: y pass (thread per (x, z)),
 // AXIS 0: x pass (thread per (y, z), rows read as aligned float4 groups).
@@ -43,7 +62,10 @@ __global__ void __launch_bounds__(B *B) k_if_pass(const float *__restrict__ in, 
     const int ob = blockIdx.x;  // output block
     const int c = blockIdx.y;
     const int a = threadIdx.x % B, b = threadIdx.x / B;
-    const int n_lo = __ldg(nbr3 + 3 * ob), n_mid = __ldg(nbr3 + 3 * ob + 1), n_hi = __ldg(nbr3 + 3 * ob + 2);
+    pdl_trigger();
+    if constexpr (AXIS != 2) pdl_wait();
+    const int n_lo = if_load<AXIS>(nbr3 + 3 * ob), n_mid = if_load<AXIS>(nbr3 + 3 * ob + 1),
+              n_hi = if_load<AXIS>(nbr3 + 3 * ob + 2);
     constexpr int W = B + 2 * RM;
     float v[W];
     if constexpr (AXIS == 0) {
@@ -55,7 +77,7 @@ __global__ void __launch_bounds__(B *B) k_if_pass(const float *__restrict__ in, 
                 const float4 *p = reinterpret_cast<const float4 *>(in + ((size_t)(n * ncomp + c) * B + b) * B * B + a * B);
 #pragma unroll
                 for (int q = 0; q < Q; q++) {
-                    const float4 w = __ldg(p + q);
+                    const float4 w = if_load<AXIS>(p + q);
                     r[4 * q] = w.x;
                     r[4 * q + 1] = w.y;
                     r[4 * q + 2] = w.z;
@@ -83,7 +105,7 @@ __global__ void __launch_bounds__(B *B) k_if_pass(const float *__restrict__ in, 
         // value at element offset q of the block at offset o: in, or ca in + cb in2
         auto val_at = [&](const float *p, size_t o, int q) -> float {
             if constexpr (EXTRA && AXIS == 2) return ca * __ldg(p + q) + cb * __ldg(in2 + o + q);
-            else return __ldg(p + q);
+            else return if_load<AXIS>(p + q);
         };
         // element (line index j along the axis) of this thread's line
         auto off = [&](int j) -> int {
@@ -120,7 +142,7 @@ __global__ void __launch_bounds__(B *B) k_if_pass(const float *__restrict__ in, 
             const float4 *ad = reinterpret_cast<const float4 *>(add + ro);
 #pragma unroll
             for (int q = 0; q < B / 4; q++) {
-                const float4 w = __ldg(ad + q);
+                const float4 w = if_load<AXIS>(ad + q);
                 r[4 * q] += w.x;
                 r[4 * q + 1] += w.y;
                 r[4 * q + 2] += w.z;
@@ -158,18 +180,18 @@ lgf_status launch3(const IfPlan &ip, int ncomp, const float *taps, const IfIO &i
     LGF_LAUNCH_CHECK("if_z_pass");
     if (P) prof->end("if_z_pass", s);
     if (P) prof->begin(s);
-    k_if_pass<B, RM, 1, false><<<dim3(ip.n2, ncomp), B * B, 0, s>>>(ip.y1, ip.y2, ip.nby, ncomp, t, nullptr, 1.f, 0.f,
-                                                                    nullptr);
-    LGF_LAUNCH_CHECK("if_y_pass");
+    const float *none = nullptr, *y1 = ip.y1, *y2 = ip.y2;
+    const int *nby = ip.nby, *nbx = ip.nbx;
+    LGF_CUDA_TRY(launch_pdl(k_if_pass<B, RM, 1, false>, dim3(ip.n2, ncomp), dim3(B * B), s, y1, ip.y2, nby, ncomp, t, none,
+                            1.f, 0.f, none));
     if (P) prof->end("if_y_pass", s);
     if (P) prof->begin(s);
     if (io.add)
-        k_if_pass<B, RM, 0, true><<<dim3(ip.n0, ncomp), B * B, 0, s>>>(ip.y2, y, ip.nbx, ncomp, t, nullptr, 1.f, 0.f,
-                                                                       io.add);
+        LGF_CUDA_TRY(launch_pdl(k_if_pass<B, RM, 0, true>, dim3(ip.n0, ncomp), dim3(B * B), s, y2, y, nbx, ncomp, t, none,
+                                1.f, 0.f, io.add));
     else
-        k_if_pass<B, RM, 0, false><<<dim3(ip.n0, ncomp), B * B, 0, s>>>(ip.y2, y, ip.nbx, ncomp, t, nullptr, 1.f, 0.f,
-                                                                        nullptr);
-    LGF_LAUNCH_CHECK("if_x_pass");
+        LGF_CUDA_TRY(launch_pdl(k_if_pass<B, RM, 0, false>, dim3(ip.n0, ncomp), dim3(B * B), s, y2, y, nbx, ncomp, t, none,
+                                1.f, 0.f, none));
     if (P) prof->end("if_x_pass", s);
     return LGF_OK;
 }

@@ -10,7 +10,12 @@
 //     1/4 sum_{m in {-1,0}} [ e^r_{n+m e_s} (f^s + f^s_{+e_q})_{n+m e_s} - e^s_{n+m e_r} (f^r + f^r_{+e_q})_{n+m e_r} ]
 //
 // One thread block per block of the set; neighbour values come through the
-// 27-neighbour table (L1/L2).
+// 27-neighbour table (L1/L2).  The operators overlap their predecessor's end (programmatic dependent
+// launch: every operator once on the 256^3 ring 123 -> 113 us) and read its output by ordinary
+// loads (__ldca), since loads through the read-only path may be taken before the wait for it.  The
+// two that follow a Poisson solve, C^T and the projection tail, do not: started beside the solve's
+// last pass they would run on its shared-memory carveout, with little L1 for the neighbours' rows
+// (the ring's step 1534 against 1428 us, its velocity refresh 748 against 739).
 #include <algorithm>
 
 #include "plan.hpp"
@@ -56,10 +61,10 @@ template <bool V4>
 __device__ __forceinline__ Quad get(const float *p)
 {
     if constexpr (V4) {
-        const float4 w = __ldg(reinterpret_cast<const float4 *>(p));
+        const float4 w = __ldca(reinterpret_cast<const float4 *>(p));
         return {{w.x, w.y, w.z, w.w}};
     } else
-        return {{__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3)}};
+        return {{__ldca(p), __ldca(p + 1), __ldca(p + 2), __ldca(p + 3)}};
 }
 template <int B, bool V4>
 struct Rows {
@@ -83,7 +88,7 @@ struct Rows {
     {
         const int dx = x < 0 ? -1 : (x >= B ? 1 : 0);
         const float *p = row(c, y, z, dx);
-        return p ? __ldg(p + x - dx * B) : 0.f;
+        return p ? __ldca(p + x - dx * B) : 0.f;
     }
     // the quad moved by one point along x
     __device__ __forceinline__ Quad next_x(const Quad &q, int c, int xq, int y, int z) const
@@ -114,6 +119,8 @@ __global__ void __launch_bounds__(Slab<B>::threads) k_op(const float *__restrict
     __shared__ int nb[27];
     if (threadIdx.x < 27) nb[threadIdx.x] = nbr27[blk * 27 + threadIdx.x];
     __syncthreads();
+    pdl_trigger();
+    pdl_wait();  // the previous kernel's output
     const int xq = threadIdx.x % S::Q, y = (threadIdx.x / S::Q) % B, z0 = threadIdx.x / (S::Q * B) * S::ZP;
     constexpr int nin = OP == 3 ? 1 : 3, nout = OP == 2 ? 1 : 3;
     const Rows<B, V4> F{in, nin, nb};
@@ -204,13 +211,15 @@ __global__ void __launch_bounds__(B *B) k_nonlinear(const float *__restrict__ in
     const int z0 = (blockIdx.x % ZS) * (B / ZS), z1 = z0 + B / ZS;
     const int x = threadIdx.x % B, y = threadIdx.x / B;
     const bool keep = out_keep == nullptr || out_keep[blk];
+    pdl_trigger();
+    pdl_wait();  // the previous kernel's output
     if (!keep) {
         for (int z = z0; z < z1; z++)
 #pragma unroll
             for (int q = 0; q < 3; q++) {
                 const size_t o = ((size_t)(blk * 3 + q) * B + z) * B * B + y * B + x;
                 out[o] = 0.f;
-                if (rv) rv[o] = __ldg(in + o);
+                if (rv) rv[o] = __ldca(in + o);
             }
         return;
     }
@@ -236,7 +245,7 @@ __global__ void __launch_bounds__(B *B) k_nonlinear(const float *__restrict__ in
             const int n = idx < H * H ? nb[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)] : -1;
             const size_t base = n >= 0 ? ((size_t)n * 3 * B + lz) * B * B + (hy - dy * B) * B + (hx - dx * B) : 0;
 #pragma unroll
-            for (int c = 0; c < 3; c++) pre[t][c] = n >= 0 ? __ldg(in + base + (size_t)c * B * B * B) + uinf[c] : 0.f;
+            for (int c = 0; c < 3; c++) pre[t][c] = n >= 0 ? __ldca(in + base + (size_t)c * B * B * B) + uinf[c] : 0.f;
         }
     };
     auto commit_f = [&](int zp) {
@@ -291,7 +300,7 @@ __global__ void __launch_bounds__(B *B) k_nonlinear(const float *__restrict__ in
             const size_t o = ((size_t)(blk * 3 + q) * B + z) * B * B + y * B + x;
             const float gv = v * 0.25f * coef;
             out[o] = gv;
-            if (rv) rv[o] = __ldg(in + o) + gv;
+            if (rv) rv[o] = __ldca(in + o) + gv;
         }
         __syncthreads();  // plane z - 1 of f and of e are no longer read
         if (z + 2 <= z1) {
@@ -318,6 +327,8 @@ __global__ void __launch_bounds__(Slab<B>::threads) k_grad_combine(const float *
     __shared__ int nb[27];
     if (threadIdx.x < 27) nb[threadIdx.x] = nbr27[blk * 27 + threadIdx.x];
     __syncthreads();
+    pdl_trigger();
+    pdl_wait();  // the previous kernel's output
     const int xq = threadIdx.x % S::Q, y = (threadIdx.x / S::Q) % B, z0 = threadIdx.x / (S::Q * B) * S::ZP;
     const Rows<B, V4> D{dhat, 1, nb};
     constexpr size_t cs = (size_t)B * B * B;
@@ -562,7 +573,10 @@ lgf_status op_launch(int op, int B, int nblk, const int *d_nbr27, const unsigned
     const bool v4 = (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
 #define LGF_OPCASE(BB, OPV)                                                                                   \
     case OPV:                                                                                                 \
-        if (v4) k_op<BB, OPV, true><<<nblk, Slab<BB>::threads, 0, s>>>(in, out, d_nbr27, inv_dx);             \
+        if (OPV != 1)                                                                                         \
+            LGF_CUDA_TRY(launch_pdl(v4 ? k_op<BB, OPV, true> : k_op<BB, OPV, false>, dim3(nblk),              \
+                                    dim3(Slab<BB>::threads), s, in, out, d_nbr27, inv_dx));                  \
+        else if (v4) k_op<BB, OPV, true><<<nblk, Slab<BB>::threads, 0, s>>>(in, out, d_nbr27, inv_dx);        \
         else k_op<BB, OPV, false><<<nblk, Slab<BB>::threads, 0, s>>>(in, out, d_nbr27, inv_dx);               \
         break;
 #define LGF_OPSWITCH(BB)                                                                                      \
@@ -572,8 +586,8 @@ lgf_status op_launch(int op, int B, int nblk, const int *d_nbr27, const unsigned
         LGF_OPCASE(BB, 2)                                                                                     \
         LGF_OPCASE(BB, 3)                                                                                     \
         case 4:                                                                                               \
-            k_nonlinear<BB><<<nblk * (BB >= 16 ? 2 : 1), BB * BB, 0, s>>>(in, out, d_nbr27, d_keep, inv_dx,   \
-                                                                           cf, u0, u1, u2, out2);             \
+            LGF_CUDA_TRY(launch_pdl(k_nonlinear<BB>, dim3(nblk * (BB >= 16 ? 2 : 1)), dim3(BB * BB), s, in,   \
+                                    out, d_nbr27, d_keep, inv_dx, cf, u0, u1, u2, out2));                     \
             break;                                                                                            \
         default: set_error("unknown operator %d", op); return LGF_ERR_ARG;                                    \
     }

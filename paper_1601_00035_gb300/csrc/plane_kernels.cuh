@@ -60,6 +60,13 @@ __device__ __forceinline__ V v_mulc(V a, C w) { return v_of(mulc(c_of(a), w)); }
 __device__ __forceinline__ V v_mul(V a, float2 w) { return v_mul(a, C{w.x, w.y}); }
 __device__ __forceinline__ V v_mulc(V a, float2 w) { return v_mulc(a, C{w.x, w.y}); }
 __device__ __forceinline__ C ld(const float2 *p) { return {p->x, p->y}; }
+// data of an earlier pass: through L2, since under programmatic dependent launch this SM's L1 may
+// still hold a line from before that pass wrote it
+__device__ __forceinline__ C ld_l2(const C *p)
+{
+    const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+    return {v.x, v.y};
+}
 
 // ---------------------------------------------------------------------------
 // in-register DFTs of length R <= 16
@@ -349,8 +356,8 @@ __device__ __forceinline__ void px_fwd_body(const PlaneGeom &g, const float *__r
         C v = {0.f, 0.f};
         if (b >= 0) {
             const float *p = src + ((size_t)((b >> 10) * g.ncomp + cc) << (3 * lB)) + ((b & 1023) << lB) + ((2 * m) & mB);
-            if (al) v = ld(reinterpret_cast<const float2 *>(p));
-            else v = {__ldg(p), __ldg(p + 1)};
+            if (al) v = ld_l2(reinterpret_cast<const C *>(p));
+            else v = {__ldcg(p), __ldcg(p + 1)};
         }
         buf[m * PX_PITCH + l] = v;
     }
@@ -419,7 +426,7 @@ __device__ __forceinline__ void px_inv_body(const PlaneGeom &g, const C *__restr
     C *col = buf + lane;
 #pragma unroll 4
     for (int k = warp; k <= M / 2; k += NW) {
-        const C u = p[(size_t)k * nrows], v = p[(size_t)(M - k) * nrows];
+        const C u = ld_l2(p + (size_t)k * nrows), v = ld_l2(p + (size_t)(M - k) * nrows);
         const C e = {0.5f * (u.x + v.x), 0.5f * (u.y - v.y)};
         const C t = {0.5f * (u.x - v.x), 0.5f * (u.y + v.y)};
         const C od = mulc(t, ld(w2 + k));
@@ -621,7 +628,7 @@ __device__ __forceinline__ void fold_rows(C *plane, const C *__restrict__ a, con
 #pragma unroll
                 for (int j = 0; j < NJ; j++) {
                     const int z = z0 + 16 * u + l16;
-                    v[u][j] = z < Ez && n + j * My < Ey ? p[j * My * Ez + z] : C{0.f, 0.f};
+                    v[u][j] = z < Ez && n + j * My < Ey ? ld_l2(p + j * My * Ez + z) : C{0.f, 0.f};
                 }
 #pragma unroll
             for (int u = 0; u < U; u++) {

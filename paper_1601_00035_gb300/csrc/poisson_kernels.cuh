@@ -72,6 +72,20 @@ __device__ __forceinline__ const double *kh_of<double>(const Geom &g) { return g
 template <typename T>
 __device__ __forceinline__ T mul_of(const Geom &g) { return sizeof(T) == 8 ? (T)g.mul64 : (T)g.mul; }
 
+// an element of the previous pass's output: through L2, since under programmatic dependent launch
+// this SM's L1 may still hold a line from before that pass wrote it
+template <typename T>
+__device__ __forceinline__ cx<T> ld_l2(const cx<T> *p)
+{
+    if constexpr (sizeof(T) == 8) {
+        const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
+        return {v.x, v.y};
+    } else {
+        const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+        return {v.x, v.y};
+    }
+}
+
 // v mod N in [0, N) for -N <= v < 2N
 template <int N>
 __device__ __forceinline__ int wrap_mod(int v)
@@ -145,7 +159,7 @@ __device__ __forceinline__ void x_fwd_body(const Geom &g, const T *__restrict__ 
                 const int blk = lut[pos >> lB];
                 if (blk >= 0) {
                     const T *p = src + ((size_t)(blk * g.ncomp + g.c0 + c) << (3 * lB)) + in_blk + (pos & mB);
-                    v[e] = {__ldg(p), __ldg(p + B)};
+                    v[e] = {__ldcg(p), __ldcg(p + B)};
                 }
             }
         }
@@ -252,7 +266,7 @@ __device__ __forceinline__ void line_body(const Geom &g, const cx<T> *__restrict
             v[e] = {(T)0, (T)0};
             const int pos = fft::in_pos<N, INV0>(e, j);
             const bool live = MODE == 2 || fft::in_lower_half<N, false>(e);
-            if (live && ok && pos < ilim) v[e] = ibase[pos * istride];
+            if (live && ok && pos < ilim) v[e] = ld_l2(ibase + pos * istride);
         }
     }
     __syncthreads();  // twiddles
@@ -395,7 +409,7 @@ __device__ __forceinline__ void zmid2_body(const Geom &g, const cx<float> *__res
         for (int e = 0; e < E; e++) {
             const int pos = fft::in_pos<N, false>(e, j);
             float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (fft::in_lower_half<N, false>(e) && ok && pos < Es2) d = ibase[pos * pstride];
+            if (fft::in_lower_half<N, false>(e) && ok && pos < Es2) d = __ldcg(ibase + pos * pstride);
             v[e] = {fft::pk2(d.x, d.z), fft::pk2(d.y, d.w)};
         }
     }
@@ -486,11 +500,11 @@ __device__ __forceinline__ void x_inv_body(const Geom &g, const cx<T> *__restric
             const int pos = fft::in_pos<N, true>(e, j);
             cx<T> a, b;
             if (pos <= N / 2) {
-                a = in[row + pos];
-                b = in[row + KX + pos];
+                a = ld_l2(in + row + pos);
+                b = ld_l2(in + row + KX + pos);
             } else {
-                a = conj(in[row + (N - pos)]);
-                b = conj(in[row + KX + (N - pos)]);
+                a = conj(ld_l2(in + row + (N - pos)));
+                b = conj(ld_l2(in + row + KX + (N - pos)));
             }
             v[e] = {a.x - b.y, a.y + b.x};
         }
