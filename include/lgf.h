@@ -109,7 +109,8 @@ typedef struct {
                            (13 row loads per 20 multiply-adds, dense over each run); 3 = quads
                            of 4 x 2 targets per warp (a source row serves two rows of targets:
                            up to 18 row loads per 40 multiply-adds; needs all 125 near offsets,
-                           else the run form) */
+                           else the run form), in shared-memory tiles of up to 48 quads where a
+                           tile holds 16 on average */
     int reserved[1];    /* must be zero */
 } lgf_plan_opts;
 

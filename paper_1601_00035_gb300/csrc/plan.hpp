@@ -233,8 +233,8 @@ struct SplitPlan {
     // sources x0 - 2 .. x0 + 5 (int4 x 4: w0..w3 | w4 s0 s1 s2 | s3..s6 | s7)
     int levels = 1;              // split levels (1: the coarse convolution is a whole-box plan)
     int nruns = 0, nrows = 0;
-    int mac_form = 0;            // the multiply-accumulate form kept: 0 pairs, 1 runs, 2 quads
-    float mac_ms[3] = {-1.f, -1.f, -1.f};  // plan-time times of the three forms (ms per launch; -1 not timed)
+    int mac_form = 0;            // the multiply-accumulate form kept: 0 pairs, 1 runs, 2 quads, 3 quads in tiles
+    float mac_ms[4] = {-1.f, -1.f, -1.f, -1.f};  // plan-time times of the forms (ms per launch; -1 not timed)
     int4 *d_run_tgt = nullptr;
     int *d_run_row = nullptr;
     int4 *d_rows = nullptr;
@@ -246,6 +246,12 @@ struct SplitPlan {
     int4 *d_quad_tgt = nullptr;
     int *d_quad_row = nullptr;
     int4 *d_qrows = nullptr;
+    // tiles of quads (k_near_mac_tiles; ntiles = 0 where a quad exceeds a tile)
+    int ntiles = 0;
+    void *d_tiles = nullptr;  // QuadTile[ntiles]
+    int *d_tile_src = nullptr;
+    uint4 *d_tile_rows = nullptr;
+    int4 *d_tile_quads = nullptr;
     // far field
     int ncsrc = 0, ncdst = 0;
     struct lgf_table *far_table = nullptr;  // G_far at even offsets (coarse octant)

@@ -444,6 +444,129 @@ __global__ void __launch_bounds__(256, 4) k_near_mac_quads(const float2 *__restr
     pdl_trigger();
 }
 
+// Quads in tiles: a thread block takes a tile of up to TILE_QUADS neighbouring quads and one chunk of
+// frequencies, and stages what they share in shared memory by bulk copies on one mbarrier: the
+// chunk's windows and the rows of the tile's source blocks (at most TILE_SRC, 256 bytes each).  The
+// direct form waits for L2 at every row-step (its table entry, then its sources: about 1650 cycles
+// each on the thin ring); here a block waits once and the other one on the SM computes meanwhile.
+// The sources a row-step does not have are skipped (three of eight are present on a thin ring), in
+// the direct form's order of summation.  Staging is repeated per tile, so the form needs many quads
+// to a tile: the thin ring's 5341 targets (24 tiles) take 1029 us against 1657 in the direct form and
+// its 2437-target coarse level 491 against 742; a dense 12^3 box (95 tiles of 6 quads) 2188 against 1327.
+// Tile sizes measured on the ring (quads, sources, threads x blocks per SM): 16, 112, 256 x 3 1239 us;
+// 16, 128, 256 x 3 1161; 32, 192, 384 x 2 1092; 48, 240, 384 x 2 1029.  240 is also what one quad can
+// reach (8 x 6 x 5 blocks), and an index fits a byte.
+// Row-step entry (uint4): x, y the tile's source indices of the eight slots (bytes); z the first
+// window rows of the two halves (low and next byte, 125 = none: the zero rows) and the presence mask (third byte).
+constexpr int TILE_QUADS = 48, TILE_SRC = 240, TILE_ROWS = 960, TILE_THREADS = 384, TILE_BLOCKS = 2;
+struct QuadTile {
+    int src0, nsrc;    // the tile's sources in tile_src
+    int row0, nrows;   // its row-steps in tile_rows
+    int quad0, nquads; // its quads in tile_quads: targets (int4 x 2), then (first, last row-step)
+};
+constexpr int TILE_WIN = 130;  // 125 windows, five zero rows
+constexpr size_t TILE_SMEM = (size_t)(TILE_WIN + TILE_SRC) * CH * sizeof(float2) + TILE_ROWS * sizeof(uint4);
+
+__global__ void __launch_bounds__(TILE_THREADS, TILE_BLOCKS) k_near_mac_tiles(const float2 *__restrict__ W, const float2 *S, int nsrc,
+                                                           const QuadTile *__restrict__ tiles,
+                                                           const int *__restrict__ tile_src,
+                                                           const uint4 *__restrict__ tile_rows,
+                                                           const int4 *__restrict__ tile_quads, int ndst, float2 *U,
+                                                           int *err)
+{
+    extern __shared__ __align__(128) unsigned char tile_sm[];
+    float2 *Kc = reinterpret_cast<float2 *>(tile_sm);             // [TILE_WIN][32]
+    float2 *Ss = Kc + TILE_WIN * CH;                                // [TILE_SRC][32]
+    uint4 *rows = reinterpret_cast<uint4 *>(Ss + TILE_SRC * CH);  // [TILE_ROWS]
+    __shared__ __align__(8) unsigned long long bar_s;
+    __shared__ int next_quad;
+    const int chunk = blockIdx.x, c = blockIdx.z, lane = threadIdx.x & 31;
+    const QuadTile t = tiles[blockIdx.y];
+    const uint32_t bar = tc::smem_addr(&bar_s);
+    if (threadIdx.x == 0) {
+        tc::mbar_init(bar, 1);
+        tc::fence_barrier_init();
+    }
+    if (threadIdx.x == 0) next_quad = 0;
+    for (int i = threadIdx.x; i < t.nrows; i += TILE_THREADS) rows[i] = __ldg(tile_rows + t.row0 + i);
+    for (int i = threadIdx.x; i < (TILE_WIN - 125) * CH; i += TILE_THREADS) Kc[125 * CH + i] = make_float2(0.f, 0.f);
+    const int my = threadIdx.x < t.nsrc ? __ldg(tile_src + t.src0 + threadIdx.x) : -1;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        tc::mbar_expect_tx(bar, (uint32_t)(125 + t.nsrc) * CH * sizeof(float2));
+        tc::bulk_g2s(tc::smem_addr(Kc), W + (size_t)chunk * 125 * CH, 125 * CH * sizeof(float2), bar);
+    }
+    __syncthreads();  // the expected byte count stands before any copy of a source row can complete
+    pdl_wait();       // the source spectra are complete
+    const float2 *Sc = S + ((size_t)c * NCHUNK + chunk) * nsrc * CH;
+    if (my >= 0) {
+        tc::fence_global_to_async();
+        tc::bulk_g2s(tc::smem_addr(Ss + threadIdx.x * CH), Sc + (size_t)my * CH, CH * sizeof(float2), bar);
+    }
+    const bool ok = tc::mbar_wait(bar, 0, STAGE_WAIT);
+    if (__syncthreads_or(!ok)) {
+        if (threadIdx.x == 0) {
+            atomicExch(err, 1);
+            tc::mbar_wait(bar, 0, STAGE_WAIT);  // let late copies land before the block exits
+        }
+        return;
+    }
+    float2 *Uc = U + ((size_t)c * NCHUNK + chunk) * ndst * CH;
+    const fft::f32x2 zero = fft::pk2(0.f, 0.f);
+    for (;;) {
+        int qi = 0;  // the next quad of the tile (quads differ in their row-steps)
+        if (lane == 0) qi = atomicAdd(&next_quad, 1);
+        qi = __shfl_sync(0xffffffffu, qi, 0);
+        if (qi >= t.nquads) break;
+        const int4 *quad = tile_quads + 3 * (t.quad0 + qi);
+        const int4 ta = __ldg(quad), tb = __ldg(quad + 1), span = __ldg(quad + 2);
+        fft::f32x2 PA[4] = {zero, zero, zero, zero}, QA[4] = {zero, zero, zero, zero};
+        fft::f32x2 PB[4] = {zero, zero, zero, zero}, QB[4] = {zero, zero, zero, zero};
+        for (int q = span.x; q < span.y; q++) {
+            const uint4 e = rows[q];
+            const uint32_t wa = e.z & 255u, wb = e.z >> 8 & 255u;
+            fft::f32x2 wA[5], wB[5];  // (the zero row for a half without targets in reach)
+#pragma unroll
+            for (int o = 0; o < 5; o++) {
+                wA[o].r = *(const unsigned long long *)(Kc + (wa + o) * CH + lane);
+                wB[o].r = *(const unsigned long long *)(Kc + (wb + o) * CH + lane);
+            }
+#pragma unroll
+            for (int k = 7; k >= 0; k--)
+                if (e.z >> (16 + k) & 1) {
+                    const float2 sv = Ss[((k < 4 ? e.x : e.y) >> (8 * (k & 3)) & 255u) * CH + lane];
+                    const fft::f32x2 sr = fft::bc2(sv.x), si = fft::bc2(sv.y);
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {  // source x0 - 2 + k = x0 + i - ox, ox = o - 2
+                        const int o = i - k + 4;
+                        if (o >= 0 && o < 5) {
+                            PA[i] = fft::fma(sr, wA[o], PA[i]);  // (Re S Re W, Re S Im W)
+                            QA[i] = fft::fma(si, wA[o], QA[i]);  // (Im S Re W, Im S Im W)
+                            PB[i] = fft::fma(sr, wB[o], PB[i]);
+                            QB[i] = fft::fma(si, wB[o], QB[i]);
+                        }
+                    }
+                }
+        }
+        const int t8[8] = {ta.x, ta.y, ta.z, ta.w, tb.x, tb.y, tb.z, tb.w};
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            float pr, pi, qr, qi2;
+            if (t8[i] >= 0) {
+                fft::unpk2(PA[i], pr, pi);
+                fft::unpk2(QA[i], qr, qi2);
+                Uc[(size_t)t8[i] * CH + lane] = make_float2(pr - qi2, pi + qr);
+            }
+            if (t8[4 + i] >= 0) {
+                fft::unpk2(PB[i], pr, pi);
+                fft::unpk2(QB[i], qr, qi2);
+                Uc[(size_t)t8[4 + i] * CH + lane] = make_float2(pr - qi2, pi + qr);
+            }
+        }
+    }
+    pdl_trigger();
+}
+
 // Inverse: one thread block per (target block, component): z, y (keeping the first
 // 16 outputs of each), then C2R in x with two rows per complex line; adds
 // mul * result (the target window of the circular convolution) to dst, which holds the
@@ -924,6 +1047,76 @@ inline int64_t key3(int x, int y, int z)
     return (((int64_t)x + off) & m) << 42 | (((int64_t)y + off) & m) << 21 | (((int64_t)z + off) & m);
 }
 
+// The quads (targets qt, two int4 each; row-steps quad_row / qrows) as tiles for k_near_mac_tiles;
+// false where a single quad has more sources or row-steps than a tile holds.
+bool build_tiles(const lgf_solve_desc &d, const std::vector<int4> &qt, const std::vector<int> &quad_row,
+                 const std::vector<int4> &qrows, std::vector<QuadTile> &tiles, std::vector<int> &tsrc,
+                 std::vector<uint4> &trows, std::vector<int4> &tquads)
+{
+    const int nq = (int)quad_row.size() - 1;
+    std::vector<std::pair<uint64_t, int>> order(nq);
+    for (int r = 0; r < nq; r++) {
+        int t = -1;
+        for (int k = 0; k < 8; k++)
+            if ((&qt[2 * (size_t)r].x)[k] >= 0) t = (&qt[2 * (size_t)r].x)[k];
+        const uint32_t p[3] = {(uint32_t)(floordiv(d.dst_blocks[3 * t], 4) + (1 << 20)),
+                               (uint32_t)(floordiv(d.dst_blocks[3 * t + 1], 2) + (1 << 20)),
+                               (uint32_t)(d.dst_blocks[3 * t + 2] + (1 << 20))};
+        uint64_t m = 0;
+        for (int b = 20; b >= 0; b--)
+            for (int a = 0; a < 3; a++) m = m << 1 | (p[a] >> b & 1);
+        order[r] = {m, r};
+    }
+    std::sort(order.begin(), order.end());
+    std::unordered_map<int, int> local;  // source block -> index in the open tile
+    auto open = [&] {
+        local.clear();
+        tiles.push_back({(int)tsrc.size(), 0, (int)trows.size(), 0, (int)(tquads.size() / 3), 0});
+    };
+    open();
+    for (const auto &o : order) {
+        const int r = o.second, n = quad_row[r + 1] - quad_row[r];
+        std::vector<int> fresh;
+        for (int pass = 0; pass < 2; pass++) {  // against the open tile, then against an empty one
+            fresh.clear();
+            std::unordered_map<int, int> seen;
+            for (int q = quad_row[r]; q < quad_row[r + 1]; q++)
+                for (int k = 0; k < 8; k++) {
+                    const int b = (&qrows[3 * (size_t)q].x)[k];
+                    if (b >= 0 && !local.count(b) && seen.emplace(b, 0).second) fresh.push_back(b);
+                }
+            const QuadTile &t = tiles.back();
+            const bool fits = t.nquads < TILE_QUADS && t.nrows + n <= TILE_ROWS && t.nsrc + (int)fresh.size() <= TILE_SRC;
+            if (fits) break;
+            if (pass == 1 || t.nquads == 0) return false;
+            open();
+        }
+        QuadTile &t = tiles.back();
+        for (int b : fresh) {
+            local.emplace(b, t.nsrc++);
+            tsrc.push_back(b);
+        }
+        tquads.push_back(qt[2 * (size_t)r]);
+        tquads.push_back(qt[2 * (size_t)r + 1]);
+        tquads.push_back(make_int4(t.nrows, t.nrows + n, 0, 0));
+        for (int q = quad_row[r]; q < quad_row[r + 1]; q++) {
+            const int *b = &qrows[3 * (size_t)q].x;
+            const int4 w = qrows[3 * (size_t)q + 2];
+            uint4 e = make_uint4(0, 0, 0, 0);
+            for (int k = 0; k < 8; k++)
+                if (b[k] >= 0) {
+                    (k < 4 ? e.x : e.y) |= (uint32_t)local[b[k]] << (8 * (k & 3));
+                    e.z |= 1u << (16 + k);
+                }
+            e.z |= (w.x < 0 ? 125u : (uint32_t)w.x) | (w.y < 0 ? 125u : (uint32_t)w.y) << 8;
+            trows.push_back(e);
+        }
+        t.nrows += n;
+        t.nquads++;
+    }
+    return true;
+}
+
 // PINT-point Lagrange weights at the midpoint of nodes PINT/2 - 1 and PINT/2 of 0 .. PINT-1
 void midpoint_weights(double w[PINT])
 {
@@ -996,6 +1189,10 @@ void free_split(SplitPlan *sp)
     cudaFree(sp->d_quad_tgt);
     cudaFree(sp->d_quad_row);
     cudaFree(sp->d_qrows);
+    cudaFree(sp->d_tiles);
+    cudaFree(sp->d_tile_src);
+    cudaFree(sp->d_tile_rows);
+    cudaFree(sp->d_tile_quads);
     cudaFree(sp->d_Q);
     cudaFree(sp->d_q);
     cudaFree(sp->d_v);
@@ -1286,6 +1483,29 @@ static lgf_status plan_split_level(lgf_plan *p, const lgf_solve_desc &d, double 
             LGF_TRY(upload_v(sp->d_quad_tgt, qt, s));
             LGF_TRY(upload_v(sp->d_quad_row, quad_row, s));
             if (!qrows.empty()) LGF_TRY(upload_v(sp->d_qrows, qrows, s));
+
+            // tiles of neighbouring quads (Morton order), cut where their sources or row-steps exceed
+            // the shared-memory limits; none where a single quad does
+            std::vector<QuadTile> tiles;
+            std::vector<int> tsrc;
+            std::vector<uint4> trows;
+            std::vector<int4> tquads;
+            if (build_tiles(d, qt, quad_row, qrows, tiles, tsrc, trows, tquads)) {
+                sp->ntiles = (int)tiles.size();
+                QuadTile *dt = nullptr;
+                LGF_TRY(dalloc_n(&dt, tiles.size(), bytes));
+                sp->d_tiles = dt;
+                LGF_TRY(dalloc_n(&sp->d_tile_src, tsrc.size(), bytes));
+                LGF_TRY(dalloc_n(&sp->d_tile_rows, trows.size(), bytes));
+                LGF_TRY(dalloc_n(&sp->d_tile_quads, tquads.size(), bytes));
+                LGF_TRY(upload_v(dt, tiles, s));
+                LGF_TRY(upload_v(sp->d_tile_src, tsrc, s));
+                LGF_TRY(upload_v(sp->d_tile_rows, trows, s));
+                LGF_TRY(upload_v(sp->d_tile_quads, tquads, s));
+                LGF_CUDA_TRY(cudaFuncSetAttribute(k_near_mac_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)TILE_SMEM));
+            }
+            LGF_CUDA_TRY(cudaStreamSynchronize(s));  // the host tables go out of scope
         }
     }
     LGF_TRY(dalloc_n(&sp->d_S, (size_t)d.ncomp * NFREQ * d.n_src, bytes));
@@ -1465,12 +1685,19 @@ lgf_status split_check(lgf_plan *p, cudaStream_t s)
 
 // The near-field multiply-accumulate in the form the plan chose (0 pairs: one target per
 // warp over its (offset, source) list; 1 runs: 4 x-adjacent targets per warp; 2 quads: 4 x 2
-// targets per warp; RUNS_PER_WARP runs or quads per warp).
+// targets per warp, RUNS_PER_WARP runs or quads per warp; 3 quads in tiles).
 constexpr int RUNS_PER_WARP = 2;
+constexpr int TILE_FILL = 16;
 static lgf_status launch_near_mac(const SplitPlan *sp, int form, cudaStream_t s)
 {
     const int nc = sp->ncomp;
-    if (form == 2)
+    if (form == 3)
+        LGF_CUDA_TRY(launch_pdl_smem(k_near_mac_tiles, dim3(NCHUNK, sp->ntiles, nc), dim3(TILE_THREADS), TILE_SMEM, s,
+                                     (const float2 *)sp->d_W, (const float2 *)sp->d_S, sp->nsrc,
+                                     (const QuadTile *)sp->d_tiles, (const int *)sp->d_tile_src,
+                                     (const uint4 *)sp->d_tile_rows, (const int4 *)sp->d_tile_quads, sp->ndst, sp->d_U,
+                                     sp->d_err));
+    else if (form == 2)
         LGF_CUDA_TRY(launch_pdl_smem(k_near_mac_quads,
                                      dim3(NCHUNK, (sp->nquads + 8 * RUNS_PER_WARP - 1) / (8 * RUNS_PER_WARP), nc),
                                      dim3(256), (size_t)sp->noff * CH * sizeof(float2), s, (const float2 *)sp->d_W,
@@ -1493,7 +1720,10 @@ static lgf_status launch_near_mac(const SplitPlan *sp, int form, cudaStream_t s)
 }
 
 // Plan time (near_form 0): time the forms (three launches each, on zeroed spectra) and keep
-// the fastest; near_form 1 / 2 / 3 takes the pair / run / quad form.  The run and quad forms
+// the fastest; near_form 1 / 2 / 3 takes the pair / run / quad form, the quads in tiles where a tile
+// holds TILE_FILL of them on average: with 16 (an 8^3 box and its neighbours) tiles take 422 us and
+// direct quads 463, with 24 (a 2^3 box and its neighbours) 12.5 and 15.2, with 18 (a 24 x 24 sheet) 82
+// and 70, with 5 (the 8^3 box alone) 288 and 186.  The run and quad forms
 // do their multiply-adds dense over each run's or quad's rows, so they win where targets fill
 // them (the 256^3 shell) and can lose where they are sparse.  The quad form needs the 125
 // offsets in canonical order (without them near_form 3 takes the run form).
@@ -1502,6 +1732,7 @@ static lgf_status choose_near_mac(SplitPlan *sp, int near_form, cudaStream_t s)
     if (near_form != 0) {  // the caller's choice
         sp->mac_form = near_form - 1;
         if (sp->mac_form == 2 && sp->nquads == 0) sp->mac_form = 1;
+        if (sp->mac_form == 2 && sp->ntiles > 0 && sp->nquads >= TILE_FILL * sp->ntiles) sp->mac_form = 3;
         return LGF_OK;
     }
     LGF_CUDA_TRY(cudaMemsetAsync(sp->d_S, 0, (size_t)sp->ncomp * NFREQ * sp->nsrc * sizeof(float2), s));
@@ -1513,7 +1744,7 @@ static lgf_status choose_near_mac(SplitPlan *sp, int near_form, cudaStream_t s)
         return LGF_ERR_CUDA;
     }
     lgf_status st = LGF_OK;
-    const int nforms = sp->nquads > 0 ? 3 : 2;
+    const int nforms = sp->ntiles > 0 ? 4 : (sp->nquads > 0 ? 3 : 2);
     for (int form = 0; form < nforms && st == LGF_OK; form++) {
         st = launch_near_mac(sp, form, s);  // warm-up
         if (st == LGF_OK && cudaEventRecord(e[0], s) != cudaSuccess) st = LGF_ERR_CUDA;
