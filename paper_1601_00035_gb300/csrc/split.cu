@@ -151,11 +151,16 @@ __global__ void k_near_pack(const double2 *__restrict__ in, int noff, float2 *__
 constexpr int SM_S1 = BN * BN * KXN;       // [z < 16][y < 16][kx]
 constexpr int SM_S2 = BN * NF * KXN;       // [z < 16][ky < 32][kx]
 constexpr size_t NEAR_SMEM = (size_t)(SM_S1 + SM_S2) * sizeof(float2);
+// Nine warps: the 544 z lines in two rounds and the 272 y lines in one (with eight, the last round held
+// 32 and 16 lines); two thread blocks per SM by the shared memory.  The thin ring: forward 76 -> 55 us
+// (1697 blocks, 236 MB written), inverse 241 -> 229 us (5341 blocks, 744 MB read: 3.3 TB/s, a block's
+// load, transform and store phases overlapped only by the other block on the SM).
+constexpr int NEAR_THREADS = 288;
 
 // Forward: one thread block per (source block, component).  R2C of the 16^3 block
 // zero-padded to 32^3: x (two real rows per complex line), y, z; the spectrum is
 // written chunked: S[((c * NCHUNK + chunk) * nsrc + b) * 32 + j].
-__global__ void __launch_bounds__(256) k_near_fwd(const float *__restrict__ src, int ncomp, int c0, int nsrc,
+__global__ void __launch_bounds__(NEAR_THREADS, 2) k_near_fwd(const float *__restrict__ src, int ncomp, int c0, int nsrc,
                                                    float2 *__restrict__ S)
 {
     extern __shared__ float2 sm[];
@@ -189,7 +194,7 @@ __global__ void __launch_bounds__(256) k_near_fwd(const float *__restrict__ src,
         }
     }
     __syncthreads();
-    for (int l = t; l < BN * KXN; l += 256) {  // y lines (z, kx)
+    for (int l = t; l < BN * KXN; l += NEAR_THREADS) {  // y lines (z, kx)
         const int z = l / KXN, kx = l % KXN;
         cx<float> a[NF];
 #pragma unroll
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(256) k_near_fwd(const float *__restrict__ src,
     __syncthreads();
     pdl_trigger();
     float2 *out = S + (size_t)c * NCHUNK * nsrc * CH;
-    for (int l = t; l < NF * KXN; l += 256) {  // z lines (ky, kx), l = ky * 17 + kx
+    for (int l = t; l < NF * KXN; l += NEAR_THREADS) {  // z lines (ky, kx), l = ky * 17 + kx
         cx<float> a[NF];
 #pragma unroll
         for (int z = 0; z < BN; z++) {
@@ -452,7 +457,7 @@ __global__ void __launch_bounds__(256, 4) k_near_mac_quads(const float2 *__restr
 // The sources a row-step does not have are skipped (three of eight are present on a thin ring), in
 // the direct form's order of summation.  Staging is repeated per tile, so the form needs many quads
 // to a tile: the thin ring's 5341 targets (24 tiles) take 1029 us against 1657 in the direct form and
-// its 2437-target coarse level 491 against 742; a dense 12^3 box (95 tiles of 6 quads) 2188 against 1327.
+// its coarse level (1830 targets) 491 against 742; a dense 12^3 box (95 tiles of 6 quads) 2188 against 1327.
 // Tile sizes measured on the ring (quads, sources, threads x blocks per SM): 16, 112, 256 x 3 1239 us;
 // 16, 128, 256 x 3 1161; 32, 192, 384 x 2 1092; 48, 240, 384 x 2 1029.  240 is also what one quad can
 // reach (8 x 6 x 5 blocks), and an index fits a byte.
@@ -571,7 +576,7 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_BLOCKS) k_near_mac_tiles(co
 // 16 outputs of each), then C2R in x with two rows per complex line; adds
 // mul * result (the target window of the circular convolution) to dst, which holds the
 // far field.
-__global__ void __launch_bounds__(256) k_near_inv(const float2 *__restrict__ U, int ndst, float *__restrict__ dst,
+__global__ void __launch_bounds__(NEAR_THREADS, 2) k_near_inv(const float2 *__restrict__ U, int ndst, float *__restrict__ dst,
                                                    int ncomp, int c0, float mul)
 {
     extern __shared__ float2 sm[];
@@ -581,7 +586,7 @@ __global__ void __launch_bounds__(256) k_near_inv(const float2 *__restrict__ U, 
     const int t = threadIdx.x;
     const float2 *in = U + (size_t)c * NCHUNK * ndst * CH;
     pdl_wait();
-    for (int l = t; l < NF * KXN; l += 256) {  // z lines (ky, kx)
+    for (int l = t; l < NF * KXN; l += NEAR_THREADS) {  // z lines (ky, kx)
         cx<float> a[NF];
 #pragma unroll
         for (int kz = 0; kz < NF; kz++) {
@@ -594,7 +599,7 @@ __global__ void __launch_bounds__(256) k_near_inv(const float2 *__restrict__ U, 
         for (int z = 0; z < BN; z++) S2[z * NF * KXN + l] = make_float2(a[z].x, a[z].y);
     }
     __syncthreads();
-    for (int l = t; l < BN * KXN; l += 256) {  // y lines (z, kx)
+    for (int l = t; l < BN * KXN; l += NEAR_THREADS) {  // y lines (z, kx)
         const int z = l / KXN, kx = l % KXN;
         cx<float> a[NF];
 #pragma unroll
@@ -641,58 +646,86 @@ __global__ void __launch_bounds__(256) k_near_inv(const float2 *__restrict__ U, 
 // 8b - 4 + l) is in constant memory.
 // ---------------------------------------------------------------------------
 __constant__ float c_P[BN * W];
-// threads per block of the two SIMT kernels: one thread block per (block, component), whose
-// three passes are short loops over the block's points; 512 threads keep every block of a
-// few-hundred-block set resident at once
-constexpr int FAR_THREADS = 512;
+// P has two kinds of rows: an even fine point 2 j takes its node j + WOFF, an odd one 2 j + 1 the ten
+// nodes j .. j + 9 with the midpoint weights.  A thread takes a whole line of 16 points / 17 nodes in
+// registers, so a line costs 80 multiply-adds and 33 shared-memory accesses (a dense 16 x 17 product
+// per output, both factors from shared memory, takes 272 and 544).  The thin ring's 5341 interpolations:
+// 217 us with the dense products, 153 with lines, 81 with the lookups ahead of the staging loads too;
+// its 1697 anterpolations: 101 and 27 us.  What bounds them now is latency between the barriers.
+constexpr int FAR_THREADS = 320;  // 289 lines of the first or last step
+__device__ __forceinline__ float mid_weight(int k) { return c_P[W + k]; }  // row 1 of P: nodes 0 .. 9
+
+// q[l] = sum_i P[i][l] f[i], the fine points in ascending order
+__device__ __forceinline__ void anterp_line(const float (&f)[BN], float (&q)[W])
+{
+#pragma unroll
+    for (int l = 0; l < W; l++) {
+        float acc = 0.f;
+#pragma unroll
+        for (int j = 0; j < BN / 2; j++) {
+            if (j == l - WOFF) acc += f[2 * j];
+            if (l - j >= 0 && l - j < PINT) acc = fmaf(mid_weight(l - j), f[2 * j + 1], acc);
+        }
+        q[l] = acc;
+    }
+}
+// f[i] = sum_l P[i][l] v[l]
+__device__ __forceinline__ void interp_line(const float (&v)[W], float (&f)[BN])
+{
+#pragma unroll
+    for (int j = 0; j < BN / 2; j++) {
+        f[2 * j] = v[j + WOFF];
+        float acc = 0.f;
+#pragma unroll
+        for (int k = 0; k < PINT; k++) acc = fmaf(mid_weight(k), v[j + k], acc);
+        f[2 * j + 1] = acc;
+    }
+}
 
 // Q_b[lz][ly][lx] = sum_i P[iz][lz] P[iy][ly] P[ix][lx] f_b[iz][iy][ix] (a W^3 window), per
 // (source block, component)
 __global__ void __launch_bounds__(FAR_THREADS) k_far_anterp(const float *__restrict__ src, int ncomp, int c0,
                                                      float *__restrict__ Q, int ncq)
 {
-    __shared__ float A[W3];
-    __shared__ float T[W3];
-    __shared__ float sP[BN * W];
+    __shared__ float A[BN * W * W];       // [z][ly][lx]
+    __shared__ float T[BN * BN * W];      // [z][y][lx]
     const int b = blockIdx.x, c = blockIdx.y, t = threadIdx.x;
     const float *f = src + ((size_t)b * ncomp + c0 + c) * (BN * BN * BN);
-    for (int i = t; i < BN * W; i += FAR_THREADS) sP[i] = c_P[i];
-    pdl_wait();
-    for (int i = t; i < BN * BN * BN; i += FAR_THREADS) A[i] = f[i];
+    for (int i = t; i < BN * BN * BN; i += FAR_THREADS) A[i / BN * W + i % BN] = f[i];  // rows at pitch W
     __syncthreads();
-    // x: T[z][y][lx] = sum_x P[x][lx] A[z][y][x]      (16 x 16 x W)
-    for (int i = t; i < BN * BN * W; i += FAR_THREADS) {
-        const int lx = i % W, row = i / W;
-        float acc = 0.f;
+    float x[BN], y[W];
+    if (t < BN * BN) {  // x: line (z, y)
 #pragma unroll
-        for (int x = 0; x < BN; x++) acc = fmaf(sP[x * W + lx], A[row * BN + x], acc);
-        T[i] = acc;
+        for (int i = 0; i < BN; i++) x[i] = A[t * W + i];
+        anterp_line(x, y);
+#pragma unroll
+        for (int l = 0; l < W; l++) T[t * W + l] = y[l];
     }
     __syncthreads();
-    // y: A[z][ly][lx] = sum_y P[y][ly] T[z][y][lx]    (16 x W x W)
-    for (int i = t; i < BN * W * W; i += FAR_THREADS) {
-        const int lx = i % W, ly = (i / W) % W, z = i / (W * W);
-        float acc = 0.f;
+    if (t < BN * W) {  // y: line (z, lx)
+        const int z = t / W, lx = t - z * W;
 #pragma unroll
-        for (int y = 0; y < BN; y++) acc = fmaf(sP[y * W + ly], T[(z * BN + y) * W + lx], acc);
-        A[i] = acc;
+        for (int i = 0; i < BN; i++) x[i] = T[(z * BN + i) * W + lx];
+        anterp_line(x, y);
+#pragma unroll
+        for (int l = 0; l < W; l++) A[(z * W + l) * W + lx] = y[l];
     }
     __syncthreads();
-    // z: Q[lz][ly][lx] = sum_z P[z][lz] A[z][ly][lx]  (W^3)
     float *out = Q + ((size_t)b * ncq + c) * W3;
-    for (int i = t; i < W3; i += FAR_THREADS) {
-        const int r = i % (W * W), lz = i / (W * W);
-        float acc = 0.f;
+    if (t < W * W) {  // z: line (ly, lx)
 #pragma unroll
-        for (int z = 0; z < BN; z++) acc = fmaf(sP[z * W + lz], A[z * W * W + r], acc);
-        out[i] = acc;
+        for (int i = 0; i < BN; i++) x[i] = A[i * W * W + t];
+        anterp_line(x, y);
+#pragma unroll
+        for (int l = 0; l < W; l++) out[l * W * W + t] = y[l];
     }
-    pdl_trigger();
 }
 
 // Coarse charges q on coarse block C: node n = 16 C + l receives Q_b[n - (8 b - 4)] from
-// each source block b whose window holds n (up to three per axis, fixed order).
-// flut: dense lookup of the fine source blocks over [fmin, fmin + fext).
+// each source block b whose window holds n (two per axis, three where n + 4 is a multiple of 8; in
+// ascending order).  flut: dense lookup of the fine source blocks over [fmin, fmin + fext); the
+// 4^3 blocks whose windows reach C (2 C - 1 .. 2 C + 2 per axis) are looked up once per thread block,
+// so that a node's loads wait for no lookup (on the thin ring 43 us; with 27 dependent ones per node 92).
 constexpr int GATHER_PARTS = 8;
 __global__ void __launch_bounds__(256) k_far_gather(const float *__restrict__ Q, int ncq,
                                                      const int *__restrict__ ccoords, const int *__restrict__ flut,
@@ -701,29 +734,38 @@ __global__ void __launch_bounds__(256) k_far_gather(const float *__restrict__ Q,
     // GATHER_PARTS thread blocks per coarse block (a slab of 16 / GATHER_PARTS planes each):
     // the coarse source blocks are few (hundreds), so one thread block each would leave
     // most SMs idle
+    __shared__ int near[64];
     const int C = blockIdx.x / GATHER_PARTS, part = blockIdx.x % GATHER_PARTS, c = blockIdx.y;
-    const int Cx = ccoords[3 * C], Cy = ccoords[3 * C + 1], Cz = ccoords[3 * C + 2];
+    if (threadIdx.x < 64) {
+        const int t = threadIdx.x;
+        const int x = 2 * ccoords[3 * C] - 1 + t % 4 - fmin.x, y = 2 * ccoords[3 * C + 1] - 1 + t / 4 % 4 - fmin.y,
+                  z = 2 * ccoords[3 * C + 2] - 1 + t / 16 - fmin.z;
+        near[t] = x >= 0 && y >= 0 && z >= 0 && x < fext.x && y < fext.y && z < fext.z
+                      ? flut[((size_t)z * fext.y + y) * fext.x + x]
+                      : -1;
+    }
     float *out = q + ((size_t)C * ncq + c) * (BN * BN * BN);
     pdl_wait();
+    __syncthreads();
     constexpr int PART = BN * BN * BN / GATHER_PARTS;
     for (int i = part * PART + threadIdx.x; i < (part + 1) * PART; i += 256) {
-        const int nx = 16 * Cx + i % BN, ny = 16 * Cy + (i / BN) % BN, nz = 16 * Cz + i / (BN * BN);
-        const int bx1 = floordiv(nx + WOFF, 8), by1 = floordiv(ny + WOFF, 8), bz1 = floordiv(nz + WOFF, 8);
+        // per axis: the last block's index in near and the node's place in its window
+        const int px = i % BN + WOFF, py = i / BN % BN + WOFF, pz = i / (BN * BN) + WOFF;
+        const int hx = px / 8 + 1, hy = py / 8 + 1, hz = pz / 8 + 1, wx = px % 8, wy = py % 8, wz = pz % 8;
         float acc = 0.f;
-        for (int dz = -2; dz <= 0; dz++) {
-            const int bz = bz1 + dz, lz = nz - (8 * bz - WOFF);
-            if (lz >= W || bz - fmin.z < 0 || bz - fmin.z >= fext.z) continue;
-            for (int dy = -2; dy <= 0; dy++) {
-                const int by = by1 + dy, ly = ny - (8 * by - WOFF);
-                if (ly >= W || by - fmin.y < 0 || by - fmin.y >= fext.y) continue;
-                for (int dx = -2; dx <= 0; dx++) {
-                    const int bx = bx1 + dx, lx = nx - (8 * bx - WOFF);
-                    if (lx >= W || bx - fmin.x < 0 || bx - fmin.x >= fext.x) continue;
-                    const int s = flut[((size_t)(bz - fmin.z) * fext.y + (by - fmin.y)) * fext.x + (bx - fmin.x)];
-                    if (s < 0) continue;
-                    acc += Q[((size_t)s * ncq + c) * W3 + (lz * W + ly) * W + lx];
-                }
+#pragma unroll
+        for (int dz = 2; dz >= 0; dz--) {
+            if (dz == 2 && wz) continue;
+            float v[9];
+#pragma unroll
+            for (int k = 0; k < 9; k++) {
+                const int dy = 2 - k / 3, dx = 2 - k % 3;
+                const bool in = (dy < 2 || wy == 0) && (dx < 2 || wx == 0);
+                const int s = in ? near[(hz - dz) * 16 + (hy - dy) * 4 + hx - dx] : -1;
+                v[k] = s >= 0 ? Q[((size_t)s * ncq + c) * W3 + ((wz + 8 * dz) * W + wy + 8 * dy) * W + wx + 8 * dx] : 0.f;
             }
+#pragma unroll
+            for (int k = 0; k < 9; k++) acc += v[k];
         }
         out[i] = acc;
     }
@@ -736,53 +778,57 @@ __global__ void __launch_bounds__(FAR_THREADS) k_far_interp(const float *__restr
                                                      const int *__restrict__ clut, int3 cmin, int3 cext,
                                                      float *__restrict__ dst, int ncomp, int c0, float mul)
 {
-    __shared__ float A[W3];
-    __shared__ float T[W3];
-    __shared__ float sP[BN * W];
+    // the window, nodes 8 b - WOFF + (0 .. 16), lies in two coarse blocks per axis: their eight are
+    // looked up once, so that the staging loads wait for no lookup
+    constexpr int AZ = BN * BN + BN;    // pitch of the lines (iy, ix): both halves of a warp on their own banks
+    __shared__ float A[W3];             // [lz][ly][lx], then [lz][iy][ix] at pitch AZ
+    __shared__ float T[W * W * W];      // [lz][ly][ix] at pitch W
+    __shared__ int near[8];
     const int b = blockIdx.x, c = blockIdx.y, t = threadIdx.x;
-    const int bx = tcoords[3 * b], by = tcoords[3 * b + 1], bz = tcoords[3 * b + 2];
-    for (int i = t; i < BN * W; i += FAR_THREADS) sP[i] = c_P[i];
-    pdl_wait();
-    for (int i = t; i < W3; i += FAR_THREADS) {
-        const int nx = 8 * bx - WOFF + i % W, ny = 8 * by - WOFF + (i / W) % W, nz = 8 * bz - WOFF + i / (W * W);
-        const int Cx = floordiv(nx, 16) - cmin.x, Cy = floordiv(ny, 16) - cmin.y, Cz = floordiv(nz, 16) - cmin.z;
-        float val = 0.f;
-        if (Cx >= 0 && Cy >= 0 && Cz >= 0 && Cx < cext.x && Cy < cext.y && Cz < cext.z) {
-            const int C = clut[((size_t)Cz * cext.y + Cy) * cext.x + Cx];
-            if (C >= 0) {
-                const int lx = nx - 16 * (Cx + cmin.x), ly = ny - 16 * (Cy + cmin.y), lz = nz - 16 * (Cz + cmin.z);
-                val = v[((size_t)C * ncv + c) * (BN * BN * BN) + (lz * BN + ly) * BN + lx];
-            }
-        }
-        A[i] = val;
+    const int n0x = 8 * tcoords[3 * b] - WOFF, n0y = 8 * tcoords[3 * b + 1] - WOFF, n0z = 8 * tcoords[3 * b + 2] - WOFF;
+    if (t < 8) {
+        const int x = floordiv(n0x, 16) + t % 2 - cmin.x, y = floordiv(n0y, 16) + t / 2 % 2 - cmin.y,
+                  z = floordiv(n0z, 16) + t / 4 - cmin.z;
+        near[t] = x >= 0 && y >= 0 && z >= 0 && x < cext.x && y < cext.y && z < cext.z
+                      ? clut[((size_t)z * cext.y + y) * cext.x + x]
+                      : -1;
     }
     __syncthreads();
-    // x: T[lz][ly][ix] = sum_lx P[ix][lx] A[lz][ly][lx]   (W x W x 16)
-    for (int i = t; i < W * W * BN; i += FAR_THREADS) {
-        const int ix = i % BN, row = i / BN;
-        float acc = 0.f;
-#pragma unroll
-        for (int l = 0; l < W; l++) acc = fmaf(sP[ix * W + l], A[row * W + l], acc);
-        T[i] = acc;
+#pragma unroll 8
+    for (int k = 0; k < (W3 + FAR_THREADS - 1) / FAR_THREADS; k++) {
+        const int i = k * FAR_THREADS + t;
+        const int x = (n0x & 15) + i % W, y = (n0y & 15) + i / W % W, z = (n0z & 15) + i / (W * W);
+        const int C = i < W3 ? near[z / 16 * 4 + y / 16 * 2 + x / 16] : -1;
+        const float val = C >= 0 ? v[((size_t)C * ncv + c) * (BN * BN * BN) + (z % 16 * BN + y % 16) * BN + x % 16] : 0.f;
+        if (i < W3) A[i] = val;
     }
     __syncthreads();
-    for (int i = t; i < W * BN * BN; i += FAR_THREADS) {  // y: A[lz][iy][ix]   (W x 16 x 16)
-        const int ix = i % BN, iy = (i / BN) % BN, lz = i / (BN * BN);
-        float acc = 0.f;
+    float x[W], y[BN];
+    if (t < W * W) {  // x: line (lz, ly)
 #pragma unroll
-        for (int l = 0; l < W; l++) acc = fmaf(sP[iy * W + l], T[(lz * W + l) * BN + ix], acc);
-        A[i] = acc;
+        for (int l = 0; l < W; l++) x[l] = A[t * W + l];
+        interp_line(x, y);
+#pragma unroll
+        for (int i = 0; i < BN; i++) T[t * W + i] = y[i];
+    }
+    __syncthreads();
+    if (t < W * BN) {  // y: line (lz, ix)
+        const int lz = t / BN, ix = t % BN;
+#pragma unroll
+        for (int l = 0; l < W; l++) x[l] = T[(lz * W + l) * W + ix];
+        interp_line(x, y);
+#pragma unroll
+        for (int i = 0; i < BN; i++) A[lz * AZ + i * BN + ix] = y[i];
     }
     __syncthreads();
     float *o = dst + ((size_t)b * ncomp + c0 + c) * (BN * BN * BN);
-    for (int i = t; i < BN * BN * BN; i += FAR_THREADS) {  // z: the far field, to which the near field is added
-        const int r = i % (BN * BN), iz = i / (BN * BN);
-        float acc = 0.f;
+    if (t < BN * BN) {  // z: line (iy, ix); the far field, to which the near field is added
 #pragma unroll
-        for (int l = 0; l < W; l++) acc = fmaf(sP[iz * W + l], A[l * BN * BN + r], acc);
-        o[i] = mul * acc;
+        for (int l = 0; l < W; l++) x[l] = A[l * AZ + t];
+        interp_line(x, y);
+#pragma unroll
+        for (int i = 0; i < BN; i++) o[i * BN * BN + t] = mul * y[i];
     }
-    pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------
@@ -1809,7 +1855,7 @@ lgf_status run_split(lgf_plan *p, const float *src, float *dst, cudaStream_t s, 
     }
     // near field: forward transforms of the source blocks, multiply-accumulate
     if (P) prof->begin(s);
-    LGF_CUDA_TRY(launch_pdl_smem(k_near_fwd, dim3(sp->nsrc, nc), dim3(256), NEAR_SMEM, s, src, nc, 0, sp->nsrc, sp->d_S));
+    LGF_CUDA_TRY(launch_pdl_smem(k_near_fwd, dim3(sp->nsrc, nc), dim3(NEAR_THREADS), NEAR_SMEM, s, src, nc, 0, sp->nsrc, sp->d_S));
     if (P) prof->end("near_fwd", s);
     if (!P) {
         LGF_CUDA_TRY(cudaEventRecord(sp->ev_src, s));
@@ -1834,7 +1880,7 @@ lgf_status run_split(lgf_plan *p, const float *src, float *dst, cudaStream_t s, 
     // near field: inverse transforms, dst += u_near
     if (!P) LGF_CUDA_TRY(cudaStreamWaitEvent(s, sp->ev_far, 0));
     if (P) prof->begin(s);
-    LGF_CUDA_TRY(launch_pdl_smem(k_near_inv, dim3(sp->ndst, nc), dim3(256), NEAR_SMEM, s, (const float2 *)sp->d_U,
+    LGF_CUDA_TRY(launch_pdl_smem(k_near_inv, dim3(sp->ndst, nc), dim3(NEAR_THREADS), NEAR_SMEM, s, (const float2 *)sp->d_U,
                                  sp->ndst, dst, nc, 0, mul_near));
     if (P) prof->end("near_inv", s);
     return LGF_OK;
