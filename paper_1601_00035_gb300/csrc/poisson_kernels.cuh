@@ -72,6 +72,17 @@ __device__ __forceinline__ const double *kh_of<double>(const Geom &g) { return g
 template <typename T>
 __device__ __forceinline__ T mul_of(const Geom &g) { return sizeof(T) == 8 ? (T)g.mul64 : (T)g.mul; }
 
+// When the next pass may begin launching: in FP32 once every block of this one has started, which hides
+// its prologue.  In FP64 only as the blocks end: an early launch spreads its blocks over what the running
+// ones leave free, two on some SMs and none on others, and at two FP64 operations per clock and SM that
+// doubled the pass (back to back, scalar: 32^3 95 us early, 41 late, 51 as plain launches; 48^3 255, 116
+// and 128; 96^3 633, 573 and 584; 128^3 1253, 1257 and 1269).
+template <typename T>
+__device__ __forceinline__ void early_trigger()
+{
+    if (sizeof(T) == 4) pdl_trigger();
+}
+
 // an element of the previous pass's output: through L2, since under programmatic dependent launch
 // this SM's L1 may still hold a line from before that pass wrote it
 template <typename T>
@@ -128,7 +139,7 @@ __device__ __forceinline__ void x_fwd_body(const Geom &g, const T *__restrict__ 
         lut_s[q] = b;
         mine |= b >= 0;
     }
-    pdl_trigger();
+    early_trigger<T>();
     pdl_wait();  // the previous pass (or the producer of src) is complete
     // twiddles, lookups; a thread block whose rows meet no source block writes
     // its zero rows without transforming them
@@ -228,7 +239,7 @@ __device__ __forceinline__ void line_body(const Geom &g, const cx<T> *__restrict
     const int i = bx * TL::LS + l;  // line p * KX + kx
     const bool ok = i < KX * line_planes<MODE>(g);
     const int Ny = g.N[1];
-    pdl_trigger();
+    early_trigger<T>();
     if constexpr (SLAB) {
         // the spectrum is fixed at plan time, so it is read before waiting on
         // the previous pass; thread (l, j) fetches kz = j, j + G, ... of line l
@@ -487,7 +498,7 @@ __device__ __forceinline__ void x_inv_body(const Geom &g, const cx<T> *__restric
     }
     // a thread block whose rows meet no target block has nothing to write
     if (!__syncthreads_or(mine)) return;
-    pdl_trigger();
+    early_trigger<T>();
     pdl_wait();  // the previous pass (or the producer of src) is complete
     const int r0 = 2 * (bx * TL::LS + l);
     const bool row_ok = r0 < nrows;
