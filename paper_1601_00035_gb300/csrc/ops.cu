@@ -187,11 +187,14 @@ __global__ void __launch_bounds__(Slab<B>::threads) k_op(const float *__restrict
     }
 }
 
-// N~(f) with shared-memory planes (replaces the per-point neighbour fetches of
-// k_op<B, 4>): thread (x, y) walks z; plane z' of f = M(u + u_inf) with a
-// one-cell halo in x and y lives in a ring of three slots, and plane z' of
-// e = C f at in-plane positions -1 .. B-1 in a ring of two, so every stencil
-// value is one shared-memory read.  Same arithmetic as eq. opr_def_nonlin.
+// N~(f) with shared-memory planes: thread (x, y) walks z; plane z' of f = M(u + u_inf) with a one-cell
+// halo in x and y lives in a ring of five slots, and plane z' of e = C f at in-plane positions
+// -1 .. B-1 in a ring of three, so every stencil value is one shared-memory read and a plane costs one
+// barrier: what a thread overtaking the others writes next lies in slots they no longer read.  The
+// planes are unrolled, so that slots are constants.  Same arithmetic as eq. opr_def_nonlin.
+// The 256^3 ring's 1251 blocks, 123 MB (184 with rv): 41 -> 33 us (48 -> 43 with rv), all of it by the
+// reads free of bank conflicts; one barrier instead of three, addresses kept, and values kept in
+// registers from plane to plane each measured the same, so what is left is latency.
 // rv (optional): also writes rv = u + out (the first stage's r = u + g without a separate
 // linear combination; the same single FP32 addition).
 template <int B>
@@ -203,21 +206,25 @@ __global__ void __launch_bounds__(B *B) k_nonlinear(const float *__restrict__ in
     constexpr int H = B + 2;  // f plane edge (halo -1 .. B)
     constexpr int HE = B + 1; // e plane edge (-1 .. B-1)
     __shared__ int nb[27];
-    __shared__ float Fs[3][3][H * H];   // [slot][component][(y+1) H + (x+1)]
-    __shared__ float Es[2][3][HE * HE]; // [slot][component][(y+1) HE + (x+1)]
-    // thread block (blk, zs) walks output planes z0 .. z1 - 1 of block blk
-    constexpr int ZS = B >= 16 ? 2 : 1;
+    __shared__ float Fs[5][3][H * H];   // [slot][component][(y+1) H + (x+1)]
+    __shared__ float Es[3][3][HE * H];  // [slot][component][(y+1) H + (x+1)], its last column unused
+    // thread block (blk, zs) walks output planes z0 .. z0 + ZP - 1 of block blk; planes are numbered from z0
+    constexpr int ZS = B >= 16 ? 2 : 1, ZP = B / ZS;
+    constexpr size_t cs = (size_t)B * B * B;
     const int blk = blockIdx.x / ZS;
-    const int z0 = (blockIdx.x % ZS) * (B / ZS), z1 = z0 + B / ZS;
-    const int x = threadIdx.x % B, y = threadIdx.x / B;
+    const int z0 = (blockIdx.x % ZS) * ZP;
+    // a warp takes rows y and y + 8 of a 16^3 block: 8 H = 16 mod 32, so its halves read different banks
+    // (adjacent rows, 18 apart, share two and cost every read a second pass)
+    const int x = threadIdx.x % B, y = B == 16 ? threadIdx.x / 32 + threadIdx.x / 16 % 2 * 8 : threadIdx.x / B;
     const bool keep = out_keep == nullptr || out_keep[blk];
+    const size_t o0 = ((size_t)blk * 3 * B + z0) * B * B + y * B + x;
     pdl_trigger();
     pdl_wait();  // the previous kernel's output
     if (!keep) {
-        for (int z = z0; z < z1; z++)
+        for (int z = 0; z < ZP; z++)
 #pragma unroll
             for (int q = 0; q < 3; q++) {
-                const size_t o = ((size_t)(blk * 3 + q) * B + z) * B * B + y * B + x;
+                const size_t o = o0 + q * cs + z * B * B;
                 out[o] = 0.f;
                 if (rv) rv[o] = __ldca(in + o);
             }
@@ -226,64 +233,73 @@ __global__ void __launch_bounds__(B *B) k_nonlinear(const float *__restrict__ in
     if (threadIdx.x < 27) nb[threadIdx.x] = nbr27[blk * 27 + threadIdx.x];
     __syncthreads();
     const float uinf[3] = {u0, u1, u2};
-    // f plane zp (-1 .. B): fetch_f reads it from global memory into registers
+    // f plane zp (-1 .. ZP): fetch_f reads it from global memory into registers
     // (each thread holds at most 2 points x 3 components: (B + 2)^2 < 2 B^2),
     // commit_f stores it into its slot, so a plane's loads can be in flight
     // while the previous plane is computed
     constexpr int PT = (H * H + B * B - 1) / (B * B);
     static_assert(PT <= 2, "halo plane points per thread");
+    int row[PT], at[PT];  // of a thread's points: neighbour (dy, dx), place in that block's plane
+#pragma unroll
+    for (int t = 0; t < PT; t++) {
+        const int idx = threadIdx.x + t * B * B;
+        const int hx = idx % H - 1, hy = idx / H - 1;
+        const int dx = hx < 0 ? -1 : (hx >= B ? 1 : 0), dy = hy < 0 ? -1 : (hy >= B ? 1 : 0);
+        row[t] = idx < H * H ? (dy + 1) * 3 + dx + 1 : -1;
+        at[t] = (hy - dy * B) * B + hx - dx * B;
+    }
     float pre[PT][3];
     auto fetch_f = [&](int zp) {
-        const int dz = zp < 0 ? -1 : (zp >= B ? 1 : 0);
-        const int lz = zp - dz * B;
+        const int z = z0 + zp, dz = z < 0 ? -1 : (z >= B ? 1 : 0);
 #pragma unroll
         for (int t = 0; t < PT; t++) {
-            const int idx = threadIdx.x + t * B * B;
-            const int hx = idx % H - 1, hy = idx / H - 1;
-            const int dx = hx < 0 ? -1 : (hx >= B ? 1 : 0);
-            const int dy = hy < 0 ? -1 : (hy >= B ? 1 : 0);
-            const int n = idx < H * H ? nb[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)] : -1;
-            const size_t base = n >= 0 ? ((size_t)n * 3 * B + lz) * B * B + (hy - dy * B) * B + (hx - dx * B) : 0;
+            const int n = row[t] >= 0 ? nb[(dz + 1) * 9 + row[t]] : -1;
+            const float *p = in + ((size_t)n * 3 * B + (z - dz * B)) * (B * B) + at[t];
 #pragma unroll
-            for (int c = 0; c < 3; c++) pre[t][c] = n >= 0 ? __ldca(in + base + (size_t)c * B * B * B) + uinf[c] : 0.f;
+            for (int c = 0; c < 3; c++) pre[t][c] = n >= 0 ? __ldca(p + c * cs) + uinf[c] : 0.f;
         }
     };
     auto commit_f = [&](int zp) {
-        float *dst = &Fs[(zp + 1) % 3][0][0];
+        float *dst = &Fs[(zp + 1) % 5][0][threadIdx.x];
 #pragma unroll
-        for (int t = 0; t < PT; t++) {
-            const int idx = threadIdx.x + t * B * B;
-            if (idx < H * H)
+        for (int t = 0; t < PT; t++)
+            if (row[t] >= 0)
 #pragma unroll
-                for (int c = 0; c < 3; c++) dst[c * H * H + idx] = pre[t][c];
-        }
+                for (int c = 0; c < 3; c++) dst[c * H * H + t * B * B] = pre[t][c];
     };
-    auto load_f = [&](int zp) {
-        fetch_f(zp);
-        commit_f(zp);
-    };
-    auto F = [&](int c, int px, int py, int pz) -> float { return Fs[(pz + 1) % 3][c][(py + 1) * H + (px + 1)]; };
-    // e plane zp (-1 .. B-1): e^c(p) = f^r(p) - f^r(p + e_s) + f^s(p + e_r) - f^s(p), (c, r, s) cyclic
+    // e plane zp (-1 .. ZP - 1): e^c(p) = f^r(p) - f^r(p + e_s) + f^s(p + e_r) - f^s(p), (c, r, s) cyclic
+    constexpr int ET = (HE * H + B * B - 1) / (B * B);
     auto make_e = [&](int zp) {
-        float *dst = &Es[(zp + 1) % 2][0][0];
-        for (int idx = threadIdx.x; idx < HE * HE; idx += B * B) {
-            const int px = idx % HE - 1, py = idx / HE - 1;
-            const float f0 = F(0, px, py, zp), f1 = F(1, px, py, zp), f2 = F(2, px, py, zp);
+        const float(*f)[H * H] = Fs[(zp + 1) % 5], (*g)[H * H] = Fs[(zp + 2) % 5];  // planes zp, zp + 1
+        float(*e)[HE * H] = Es[(zp + 1) % 3];
+#pragma unroll
+        for (int t = 0; t < ET; t++) {
+            const int p = threadIdx.x + t * B * B;
+            if (p >= HE * H) continue;
+            const float f0 = f[0][p], f1 = f[1][p], f2 = f[2][p];
             // c = 0 (r = y, s = z); c = 1 (r = z, s = x); c = 2 (r = x, s = y)
-            dst[0 * HE * HE + idx] = (f1 - F(1, px, py, zp + 1) + F(2, px, py + 1, zp) - f2) * inv_dx;
-            dst[1 * HE * HE + idx] = (f2 - F(2, px + 1, py, zp) + F(0, px, py, zp + 1) - f0) * inv_dx;
-            dst[2 * HE * HE + idx] = (f0 - F(0, px, py + 1, zp) + F(1, px + 1, py, zp) - f1) * inv_dx;
+            e[0][p] = (f1 - g[1][p] + f[2][p + H] - f2) * inv_dx;
+            e[1][p] = (f2 - f[2][p + 1] + g[0][p] - f0) * inv_dx;
+            e[2][p] = (f0 - f[0][p + H] + f[1][p + 1] - f1) * inv_dx;
         }
     };
-    auto Ev = [&](int c, int px, int py, int pz) -> float { return Es[(pz + 1) % 2][c][(py + 1) * HE + (px + 1)]; };
-    load_f(z0 - 1);
-    load_f(z0);
-    load_f(z0 + 1);
+    const int pf = (y + 1) * H + x + 1;
+    auto F = [&](int c, int dx, int dy, int zp) -> float { return Fs[(zp + 1) % 5][c][pf + dy * H + dx]; };
+    auto Ev = [&](int c, int dx, int dy, int zp) -> float { return Es[(zp + 1) % 3][c][pf + dy * H + dx]; };
+    fetch_f(-1);
+    commit_f(-1);
+    fetch_f(0);
+    commit_f(0);
+    fetch_f(1);
+    commit_f(1);
     __syncthreads();
-    make_e(z0 - 1);
-    fetch_f(z0 + 2);  // B / ZS >= 8
-    for (int z = z0; z < z1; z++) {
-        make_e(z);  // reads f planes z, z + 1
+    make_e(-1);
+    fetch_f(2);  // ZP >= 2
+#pragma unroll
+    for (int z = 0; z < ZP; z++) {
+        if (z + 2 <= ZP) commit_f(z + 2);  // the slot of plane z - 3
+        if (z + 3 <= ZP) fetch_f(z + 3);   // in flight during this plane
+        make_e(z);                         // reads f planes z, z + 1; the slot of plane z - 3
         __syncthreads();
         const int o[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};  // unit offsets e_q
 #pragma unroll
@@ -292,22 +308,16 @@ __global__ void __launch_bounds__(B *B) k_nonlinear(const float *__restrict__ in
             float v = 0.f;
 #pragma unroll
             for (int m = -1; m <= 0; m++) {
-                const int ax = x + m * o[s2][0], ay = y + m * o[s2][1], az = z + m * o[s2][2];
+                const int ax = m * o[s2][0], ay = m * o[s2][1], az = z + m * o[s2][2];
                 v += Ev(r, ax, ay, az) * (F(s2, ax, ay, az) + F(s2, ax + o[q][0], ay + o[q][1], az + o[q][2]));
-                const int bx = x + m * o[r][0], by = y + m * o[r][1], bz = z + m * o[r][2];
+                const int bx = m * o[r][0], by = m * o[r][1], bz = z + m * o[r][2];
                 v -= Ev(s2, bx, by, bz) * (F(r, bx, by, bz) + F(r, bx + o[q][0], by + o[q][1], bz + o[q][2]));
             }
-            const size_t o = ((size_t)(blk * 3 + q) * B + z) * B * B + y * B + x;
+            const size_t i = o0 + q * cs + z * B * B;
             const float gv = v * 0.25f * coef;
-            out[o] = gv;
-            if (rv) rv[o] = __ldca(in + o) + gv;
+            out[i] = gv;
+            if (rv) rv[i] = __ldca(in + i) + gv;
         }
-        __syncthreads();  // plane z - 1 of f and of e are no longer read
-        if (z + 2 <= z1) {
-            commit_f(z + 2);                   // into plane z - 1's slot
-            if (z + 3 <= z1) fetch_f(z + 3);   // in flight during plane z + 1
-        }
-        __syncthreads();
     }
 }
 
