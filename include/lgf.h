@@ -186,9 +186,11 @@ lgf_status lgf_plan_workspace_bytes(const lgf_plan *p, size_t *bytes);
 
 /* Poisson: for every solve i, dst[i] (device, [n_dst][ncomp][B^3] FP32,
  * overwritten on every target point) = scale * dx^2 * G * src[i] (device,
- * [n_src][ncomp][B^3] FP32).  Asynchronous on `stream`; no allocation.  A
- * plan with more than one (solve, component) unit runs the units on its own
- * worker streams, forked from and joined back to `stream` with events; with
+ * [n_src][ncomp][B^3] FP32).  Asynchronous on `stream`; no allocation.  One
+ * solve in the three-pass form runs all its components in each launch on
+ * `stream`; other plans with more than one (solve, component) unit run the
+ * units on their own worker streams, forked from and joined back to `stream`
+ * with events; with
  * opts->use_graph the whole sequence is captured once per set of buffers
  * and replayed.  dst[i] may be the buffer src[i] for a solve with ncomp = 1
  * (every source value is read before the first result is written; the
