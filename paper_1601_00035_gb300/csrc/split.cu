@@ -461,6 +461,7 @@ __global__ void __launch_bounds__(256, 4) k_near_mac_quads(const float2 *__restr
 // Tile sizes measured on the ring (quads, sources, threads x blocks per SM): 16, 112, 256 x 3 1239 us;
 // 16, 128, 256 x 3 1161; 32, 192, 384 x 2 1092; 48, 240, 384 x 2 1029.  240 is also what one quad can
 // reach (8 x 6 x 5 blocks), and an index fits a byte.
+// What bounds it now is shared memory, 72 % of the cycles: ten window rows of two wavefronts per row-step.
 // Row-step entry (uint4): x, y the tile's source indices of the eight slots (bytes); z the first
 // window rows of the two halves (low and next byte, 125 = none: the zero rows) and the presence mask (third byte).
 constexpr int TILE_QUADS = 48, TILE_SRC = 240, TILE_ROWS = 960, TILE_THREADS = 384, TILE_BLOCKS = 2;
