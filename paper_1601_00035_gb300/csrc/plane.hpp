@@ -6,6 +6,7 @@
 // against the five passes of poisson.cu (which FP64 plans and boxes beyond the lengths here keep).
 #pragma once
 #include "plan.hpp"
+#include "plane_len.hpp"
 
 namespace lgf {
 
@@ -55,21 +56,5 @@ struct PlaneYZ {
     static lgf_status grp(const PlaneTask *t, const int *cta, int ncta, size_t smem, int threads, int Dy,
                           cudaStream_t s);
 };
-
-// radices of M = R1 * R2 (R2 even)
-__host__ __device__ constexpr int plane_r2(int M)
-{
-    return M <= 32 ? 4 : M == 48 ? 6 : M <= 128 ? 8 : M == 144 ? 12 : M == 160 ? 10 : M == 192 ? 12 : M == 224 ? 14 : 16;
-}
-__host__ __device__ constexpr int plane_r1(int M) { return M / plane_r2(M); }
-// the z transform's second radix (even), and the threads per SM its registers leave room for
-__host__ __device__ constexpr int plane_z2(int M)
-{
-    return M == 16 ? 4 : (M <= 80 ? 8 : 16);
-}
-__host__ __device__ constexpr int plane_yz_threads(int M) { return M <= 128 ? 1024 : M <= 192 ? 768 : 512; }
-
-#define LGF_PLANE_LENGTHS(X) \
-    X(16) X(32) X(48) X(64) X(80) X(96) X(112) X(128) X(144) X(160) X(176) X(192) X(208) X(224) X(240) X(256)
 
 }  // namespace lgf

@@ -593,16 +593,15 @@ __device__ __forceinline__ void z_mid(C *p, const float (&kv)[YZ<MZ>::R2], const
         v_st(p + k2, a[k2]);
     }
 }
-// its spectrum values: frequency kk = q + R1 k2 of a half folds to kk below Mz / 2 (k2 < R2 / 2) and
-// to Mz - kk (even half) or Mz - 1 - kk (odd) above.  K: the spectrum of the thread block's plane,
-// col: the column's place in its rows of My.
+// its spectrum values (rows: plane_len.hpp).  K: the spectrum of the thread block's plane, col: the
+// column's place in its rows of My.
 template <int MZ>
 __device__ __forceinline__ void z_spectrum(float (&kv)[YZ<MZ>::R2], const float *K, unsigned col, unsigned My, bool odd,
                                            int q)
 {
     constexpr int R1 = YZ<MZ>::R1, R2 = YZ<MZ>::R2;
-    const unsigned lo = col + ((odd ? MZ / 2 + 1 : 0) + q) * My;
-    const unsigned hi = col + ((odd ? MZ / 2 + MZ : MZ) - q) * My;
+    const unsigned lo = col + plane_row_lo(MZ, odd, q) * My;
+    const unsigned hi = col + plane_row_hi(MZ, odd, q) * My;
 #pragma unroll
     for (int k2 = 0; k2 < R2; k2++) kv[k2] = k2 < R2 / 2 ? __ldg(K + (lo + k2 * R1 * My)) : __ldg(K + (hi - k2 * R1 * My));
 }
@@ -724,7 +723,7 @@ __device__ __forceinline__ void yz_body(const PlaneGeom &g, const C *__restrict_
             C *colp = plane + col * P;
             float kv[R2];
             // the first middle butterfly's spectrum, in flight during the first stage
-            z_spectrum<MZ>(kv, Kp, col, My, b >= R1, b >= R1 ? b - R1 : b);
+            if (plane_mid_any(MZ, b)) z_spectrum<MZ>(kv, Kp, col, My, b >= R1, b >= R1 ? b - R1 : b);
             {
                 V x[R1], v[R1];
 #pragma unroll
