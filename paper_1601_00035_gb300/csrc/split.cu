@@ -146,7 +146,10 @@ __global__ void k_near_pack(const double2 *__restrict__ in, int noff, float2 *__
 }
 
 // ---------------------------------------------------------------------------
-// Near field, per execution.
+// Near field, per execution.  The kernels start while their predecessor on the stream drains, and so
+// read what an earlier kernel wrote (src, S, U; in the far field src and the coarse potential) by
+// ordinary loads (__ldca) behind pdl_wait: a plain load of a const __restrict__ array may become one
+// through the read-only path, which may be taken before the wait.
 // ---------------------------------------------------------------------------
 constexpr int SM_S1 = BN * BN * KXN;       // [z < 16][y < 16][kx]
 constexpr int SM_S2 = BN * NF * KXN;       // [z < 16][ky < 32][kx]
@@ -176,7 +179,7 @@ __global__ void __launch_bounds__(NEAR_THREADS, 2) k_near_fwd(const float *__res
         const float4 *r1 = reinterpret_cast<const float4 *>(f + (2 * t + 1) * BN);
 #pragma unroll
         for (int i = 0; i < 4; i++) {
-            const float4 u = r0[i], v = r1[i];
+            const float4 u = __ldca(r0 + i), v = __ldca(r1 + i);
             a[4 * i + 0] = {u.x, v.x};
             a[4 * i + 1] = {u.y, v.y};
             a[4 * i + 2] = {u.z, v.z};
@@ -286,7 +289,7 @@ __global__ void __launch_bounds__(256) k_near_mac(const float2 *__restrict__ W, 
             for (int k = 0; k < n; k++) {
                 const int d = __shfl_sync(0xffffffffu, my.x, k);
                 const int s = __shfl_sync(0xffffffffu, my.y, k);
-                const float2 sv = Sc[(size_t)s * CH + lane];
+                const float2 sv = __ldca(Sc + (size_t)s * CH + lane);
                 const float2 kv = Kc[d * CH + lane];
                 ar = fmaf(kv.x, sv.x, ar);
                 ar = fmaf(-kv.y, sv.y, ar);
@@ -338,7 +341,7 @@ __global__ void __launch_bounds__(256) k_near_mac_runs(const float2 *__restrict_
             fft::f32x2 sr[8], si[8];
 #pragma unroll
             for (int k = 0; k < 8; k++) {
-                const float2 v = src[k] >= 0 ? Sc[(size_t)src[k] * CH + lane] : make_float2(0.f, 0.f);
+                const float2 v = src[k] >= 0 ? __ldca(Sc + (size_t)src[k] * CH + lane) : make_float2(0.f, 0.f);
                 sr[k] = fft::bc2(v.x);
                 si[k] = fft::bc2(v.y);
             }
@@ -400,7 +403,7 @@ __global__ void __launch_bounds__(256, 4) k_near_mac_quads(const float2 *__restr
             fft::f32x2 sr[8], si[8];
 #pragma unroll
             for (int k = 0; k < 8; k++) {
-                const float2 v = src[k] >= 0 ? Sc[(size_t)src[k] * CH + lane] : make_float2(0.f, 0.f);
+                const float2 v = src[k] >= 0 ? __ldca(Sc + (size_t)src[k] * CH + lane) : make_float2(0.f, 0.f);
                 sr[k] = fft::bc2(v.x);
                 si[k] = fft::bc2(v.y);
             }
@@ -592,7 +595,7 @@ __global__ void __launch_bounds__(NEAR_THREADS, 2) k_near_inv(const float2 *__re
 #pragma unroll
         for (int kz = 0; kz < NF; kz++) {
             const int fq = kz * (NF * KXN) + l;
-            const float2 v = in[((size_t)(fq / CH) * ndst + b) * CH + (fq % CH)];
+            const float2 v = __ldca(in + ((size_t)(fq / CH) * ndst + b) * CH + (fq % CH));
             a[kz] = {v.x, v.y};
         }
         fft::dft_reg<NF, true, float, 0, false>(a);
@@ -951,7 +954,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_far_anterp_tc(const float *__res
     tc_setup<16>(sm, Bhl);
     const float *f = src + ((size_t)b * ncomp + c0 + c) * (BN * BN * BN);
     pdl_wait();
-    for (int i = t; i < BN * BN * BN; i += TC_THREADS) tc_put<16>(sm, i / BN, i % BN, f[i]);  // rows (z, y), k = x
+    for (int i = t; i < BN * BN * BN; i += TC_THREADS) tc_put<16>(sm, i / BN, i % BN, __ldca(f + i));  // rows (z, y), k = x
     uint32_t ph = 0;
     bool ok = tc_pass<16, 32>(sm, 2, ph);
     float v[32];
@@ -1009,7 +1012,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_far_interp_tc(const float *__res
             const int C = clut[((size_t)Cz * cext.y + Cy) * cext.x + Cx];
             if (C >= 0) {
                 const int lx = nx - 16 * (Cx + cmin.x), ly = ny - 16 * (Cy + cmin.y), lz = nz - 16 * (Cz + cmin.z);
-                val = vc[((size_t)C * ncv + c) * (BN * BN * BN) + (lz * BN + ly) * BN + lx];
+                val = __ldca(vc + ((size_t)C * ncv + c) * (BN * BN * BN) + (lz * BN + ly) * BN + lx);
             }
         }
         tc_put<24>(sm, i / W, i % W, val);
