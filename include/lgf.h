@@ -109,8 +109,8 @@ typedef struct {
                            (13 row loads per 20 multiply-adds, dense over each run); 3 = quads
                            of 4 x 2 targets per warp (a source row serves two rows of targets:
                            up to 18 row loads per 40 multiply-adds; needs all 125 near offsets,
-                           else the run form), in shared-memory tiles of up to 48 quads where a
-                           tile holds 16 on average */
+                           else the run form), in shared-memory tiles of up to 48 quads where
+                           the work of a tile outweighs its staging */
     int reserved[1];    /* must be zero */
 } lgf_plan_opts;
 
@@ -166,6 +166,11 @@ lgf_status lgf_conv_plan(const lgf_table *t, const lgf_solve_desc *solves, int n
  * an autotuned plan (opts->method = 2), *ms_whole_box and *ms_split receive the device times
  * of the two candidates measured at plan time (-1 where not timed); either pointer may be NULL. */
 int lgf_plan_method(const lgf_plan *p, double *ms_whole_box, double *ms_split);
+
+/* The near-field form that a split plan executes: 1 pairs, 2 runs, 3 quads, 4 quads in
+ * shared-memory tiles (opts->near_form = 3 takes 3 or 4); 0 for a whole-box plan, -1 for NULL.
+ * ms (may be NULL): ms[i] receives the time of form i + 1 measured at plan time (-1 where not timed). */
+int lgf_plan_near_form(const lgf_plan *p, double ms[4]);
 
 /* Synchronises `stream` and reports LGF_ERR_TIMEOUT if a bounded device-side wait of the
  * plan's kernels gave up since the last check (the flag is then cleared; the results of

@@ -1040,6 +1040,16 @@ int lgf_plan_method(const lgf_plan *p, double *ms_whole_box, double *ms_split)
     return p->method;
 }
 
+int lgf_plan_near_form(const lgf_plan *p, double ms[4])
+{
+    if (!p) return -1;
+    if (p->sub) return lgf_plan_near_form(p->sub, ms);
+    const SplitPlan *sp = p->split;
+    if (ms)
+        for (int i = 0; i < 4; i++) ms[i] = sp ? sp->mac_ms[i] : -1.0;
+    return sp ? sp->mac_form + 1 : 0;
+}
+
 lgf_status lgf_plan_workspace_bytes(const lgf_plan *p, size_t *bytes)
 {
     clear_error();

@@ -248,6 +248,7 @@ struct SplitPlan {
     int4 *d_qrows = nullptr;
     // tiles of quads (k_near_mac_tiles; ntiles = 0 where a quad exceeds a tile)
     int ntiles = 0;
+    bool tiles_pay = false;  // near_form 3 takes the tiles
     void *d_tiles = nullptr;  // QuadTile[ntiles]
     int *d_tile_src = nullptr;
     uint4 *d_tile_rows = nullptr;

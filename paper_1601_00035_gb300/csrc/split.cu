@@ -458,9 +458,10 @@ __global__ void __launch_bounds__(256, 4) k_near_mac_quads(const float2 *__restr
 // direct form waits for L2 at every row-step (its table entry, then its sources: about 1650 cycles
 // each on the thin ring); here a block waits once and the other one on the SM computes meanwhile.
 // The sources a row-step does not have are skipped (three of eight are present on a thin ring), in
-// the direct form's order of summation.  Staging is repeated per tile, so the form needs many quads
-// to a tile: the thin ring's 5341 targets (24 tiles) take 1029 us against 1657 in the direct form and
-// its coarse level (1830 targets) 491 against 742; a dense 12^3 box (95 tiles of 6 quads) 2188 against 1327.
+// the direct form's order of summation.  Staging is repeated per tile, so the form needs many row-steps
+// to what a tile stages (tiles_pay): the thin ring's 5341 targets (24 tiles) take 1029 us against 1657 in
+// the direct form and its coarse level (1830 targets) 491 against 742; a dense 12^3 box and its
+// neighbours (95 tiles of 6 quads) 2183 against 1621.
 // Tile sizes measured on the ring (quads, sources, threads x blocks per SM): 16, 112, 256 x 3 1239 us;
 // 16, 128, 256 x 3 1161; 32, 192, 384 x 2 1092; 48, 240, 384 x 2 1029.  240 is also what one quad can
 // reach (8 x 6 x 5 blocks), and an index fits a byte.
@@ -473,6 +474,15 @@ struct QuadTile {
     int row0, nrows;   // its row-steps in tile_rows
     int quad0, nquads; // its quads in tile_quads: targets (int4 x 2), then (first, last row-step)
 };
+// Whether the tiles are the faster of the two quad forms: a tile costs the direct form's work with its
+// waits hidden, and on top the staging of 125 window rows and its sources, so what counts is the
+// row-steps per staged row.  Measured over 77 block sets (boxes, sheets, columns, rings, random and
+// scattered sets): time in tiles over time in direct quads 1.02 to 2.2 up to 0.33 row-steps per staged
+// row (a 24 x 24 sheet 0.29: 82 against 79 us; an 8^3 box 0.33: 286 and 237; exceptions 0.82 to 0.95 on
+// three small sets), 0.75 to 1.04 between 0.43 and 0.53 (random blocks at 60 % 0.48: 1248 and 1397), 0.85
+// down to 0.35 from 0.57 on (an 8^3 box with its neighbours 0.72: 422 and 580; the thin rings 1.5 to 2).
+// The quads in a tile alone do not tell: the sheet has 18, that 60 % set 7.
+bool tiles_pay(size_t ntiles, size_t nrows, size_t nsrc) { return 5 * nrows >= 2 * (125 * ntiles + nsrc); }
 constexpr int TILE_WIN = 130;  // 125 windows, five zero rows
 constexpr size_t TILE_SMEM = (size_t)(TILE_WIN + TILE_SRC) * CH * sizeof(float2) + TILE_ROWS * sizeof(uint4);
 
@@ -1542,6 +1552,7 @@ static lgf_status plan_split_level(lgf_plan *p, const lgf_solve_desc &d, double 
             std::vector<int4> tquads;
             if (build_tiles(d, qt, quad_row, qrows, tiles, tsrc, trows, tquads)) {
                 sp->ntiles = (int)tiles.size();
+                sp->tiles_pay = tiles_pay(tiles.size(), trows.size(), tsrc.size());
                 QuadTile *dt = nullptr;
                 LGF_TRY(dalloc_n(&dt, tiles.size(), bytes));
                 sp->d_tiles = dt;
@@ -1737,7 +1748,6 @@ lgf_status split_check(lgf_plan *p, cudaStream_t s)
 // warp over its (offset, source) list; 1 runs: 4 x-adjacent targets per warp; 2 quads: 4 x 2
 // targets per warp, RUNS_PER_WARP runs or quads per warp; 3 quads in tiles).
 constexpr int RUNS_PER_WARP = 2;
-constexpr int TILE_FILL = 16;
 static lgf_status launch_near_mac(const SplitPlan *sp, int form, cudaStream_t s)
 {
     const int nc = sp->ncomp;
@@ -1770,11 +1780,8 @@ static lgf_status launch_near_mac(const SplitPlan *sp, int form, cudaStream_t s)
 }
 
 // Plan time (near_form 0): time the forms (three launches each, on zeroed spectra) and keep
-// the fastest; near_form 1 / 2 / 3 takes the pair / run / quad form, the quads in tiles where a tile
-// holds TILE_FILL of them on average: with 16 (an 8^3 box and its neighbours) tiles take 422 us and
-// direct quads 463, with 24 (a 2^3 box and its neighbours) 12.5 and 15.2, with 18 (a 24 x 24 sheet) 82
-// and 70, with 5 (the 8^3 box alone) 288 and 186.  The run and quad forms
-// do their multiply-adds dense over each run's or quad's rows, so they win where targets fill
+// the fastest; near_form 1 / 2 / 3 takes the pair / run / quad form, the quads in tiles where tiles_pay.
+// The run and quad forms do their multiply-adds dense over each run's or quad's rows, so they win where targets fill
 // them (the 256^3 shell) and can lose where they are sparse.  The quad form needs the 125
 // offsets in canonical order (without them near_form 3 takes the run form).
 static lgf_status choose_near_mac(SplitPlan *sp, int near_form, cudaStream_t s)
@@ -1782,7 +1789,7 @@ static lgf_status choose_near_mac(SplitPlan *sp, int near_form, cudaStream_t s)
     if (near_form != 0) {  // the caller's choice
         sp->mac_form = near_form - 1;
         if (sp->mac_form == 2 && sp->nquads == 0) sp->mac_form = 1;
-        if (sp->mac_form == 2 && sp->ntiles > 0 && sp->nquads >= TILE_FILL * sp->ntiles) sp->mac_form = 3;
+        if (sp->mac_form == 2 && sp->tiles_pay) sp->mac_form = 3;
         return LGF_OK;
     }
     LGF_CUDA_TRY(cudaMemsetAsync(sp->d_S, 0, (size_t)sp->ncomp * NFREQ * sp->nsrc * sizeof(float2), s));

@@ -88,6 +88,7 @@ _SIGS = {
     "lgf_plan_workspace_bytes": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_size_t)]),
     "lgf_plan_method": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_double),
                                        ctypes.POINTER(ctypes.c_double)]),
+    "lgf_plan_near_form": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_double)]),
     "lgf_plan_check": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     "lgf_wait_probe": (ctypes.c_int, [ctypes.c_int, ctypes.c_void_p]),
     "lgf_conv_execute": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_void_p),
@@ -255,6 +256,12 @@ class Plan:
         a, b = ctypes.c_double(), ctypes.c_double()
         m = load().lgf_plan_method(self._h, ctypes.byref(a), ctypes.byref(b))
         return m, a.value, b.value
+
+    def near_form(self):
+        """(near-field form of a split plan: 1 pairs, 2 runs, 3 quads, 4 quads in tiles; 0 whole box,
+        plan-time ms of the four forms, -1 where not timed)."""
+        ms = (ctypes.c_double * 4)()
+        return load().lgf_plan_near_form(self._h, ms), list(ms)
 
     def check(self, stream=None):
         """Synchronise and raise LGFError(LGF_ERR_TIMEOUT) if a bounded device wait gave up."""
