@@ -103,8 +103,12 @@ struct Roots {
     }
 };
 
-// odd length Q by the symmetric sums x_m + x_(Q-m), x_m - x_(Q-m)
-template <int Q, bool INV>
+// Odd length Q by the symmetric sums x_m + x_(Q-m), x_m - x_(Q-m).  A smooth field's spectrum lies in
+// the lowest frequencies, in an inverse transform x_0 and x_(+-1) and, behind the index map of a
+// prime-factor product (UP), x_0 and x_(+-H).  Those come last, so that the partial sums that are
+// rounded stay small: from x_0 on, the point differences along x of a 200 x 16 x 16 solve (13-point
+// sums) were off by 5.9e-6 relative, in this order by 5.1e-6 (the five passes: 4.8e-6); same time.
+template <int Q, bool INV, bool UP = false>
 __device__ __forceinline__ void dft_sym(V (&x)[Q])
 {
     constexpr Roots<Q> W{};
@@ -116,19 +120,21 @@ __device__ __forceinline__ void dft_sym(V (&x)[Q])
         d[m] = x[m + 1] - x[Q - 1 - m];
     }
     const V x0 = x[0];
-    V s = x0;
+    V s = t[UP ? 0 : H - 1];
 #pragma unroll
-    for (int m = 0; m < H; m++) s = s + t[m];
-    x[0] = s;
+    for (int i = 1; i < H; i++) s = s + t[UP ? i : H - 1 - i];
+    x[0] = s + x0;
 #pragma unroll
     for (int k = 1; k <= H; k++) {
-        V a = x0, b = V{kZero};
+        V a, b;
 #pragma unroll
-        for (int m = 1; m <= H; m++) {
+        for (int i = 0; i < H; i++) {
+            const int m = UP ? i + 1 : H - i;
             const V c = fft::bc2((float)W.c[(k * m) % Q]), sn = fft::bc2((float)W.s[(k * m) % Q]);
-            a = fft::fma(c, t[m - 1], a);
-            b = m == 1 ? sn * d[0] : fft::fma(sn, d[m - 1], b);
+            a = i == 0 ? c * t[m - 1] : fft::fma(c, t[m - 1], a);
+            b = i == 0 ? sn * d[m - 1] : fft::fma(sn, d[m - 1], b);
         }
+        a = a + x0;
         x[k] = INV ? add_i(a, b) : sub_i(a, b);
         x[Q - k] = INV ? sub_i(a, b) : add_i(a, b);
     }
@@ -237,8 +243,8 @@ __device__ __forceinline__ void dft(V (&a)[R])
             u[0][n2] = p + q;
             u[1][n2] = p - q;
         }
-        dft_sym<Q, INV>(u[0]);
-        dft_sym<Q, INV>(u[1]);
+        dft_sym<Q, INV, true>(u[0]);
+        dft_sym<Q, INV, true>(u[1]);
 #pragma unroll
         for (int k1 = 0; k1 < 2; k1++)
 #pragma unroll
@@ -254,7 +260,7 @@ __device__ __forceinline__ void dft(V (&a)[R])
         }
 #pragma unroll
         for (int k1 = 0; k1 < 3; k1++) {
-            dft_sym<5, INV>(u[k1]);
+            dft_sym<5, INV, true>(u[k1]);
 #pragma unroll
             for (int k2 = 0; k2 < 5; k2++) a[(10 * k1 + 6 * k2) % 15] = u[k1][k2];
         }
