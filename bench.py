@@ -145,24 +145,19 @@ def pass_bytes(plan_geom):
     X3 = nc * Et[2] * N[1] * KX * 8
     X4 = nc * Et[2] * Et[1] * KX * 8
     Kh = (N[0] // 2 + 1) * (N[1] // 2 + 1) * (N[2] // 2 + 1) * 4
+    Kt = (N[0] // 2 + 1) * N[1] * (N[2] // 2 + 1) * 4  # three-pass form: all of y
     src = g["nsrc"] * nc * B ** 3 * 4
     dst = g["ndst"] * nc * B ** 3 * 4
     return {"x_fwd_gather_r2c": src + X1, "y_fwd": X1 + X2, "z_fwd_mul_inv": X2 + Kh + X3, "y_inv": X3 + X4,
-            "yz_conv": X1 + Kh + X4, "x_inv_c2r_scatter": X4 + dst}
+            "yz_conv": X1 + Kt + X4, "x_inv_c2r_scatter": X4 + dst}
 
 
-def geometry(src_c, dst_c, ncomp):
-    from paper_1601_00035_gb300.lgf import fft_length
+def geometry(src_c, dst_c, ncomp, lengths):
+    """Boxes, block counts and the FFT lengths (x, y, z) that the plan runs on."""
     s, t = np.asarray(src_c), np.asarray(dst_c)
     Es = [int((s[:, a].max() - s[:, a].min() + 1) * B) for a in range(3)]
     Et = [int((t[:, a].max() - t[:, a].min() + 1) * B) for a in range(3)]
-    N = []
-    for a in range(3):
-        S0, S1 = s[:, a].min() * B, (s[:, a].max() + 1) * B - 1
-        T0, T1 = t[:, a].min() * B, (t[:, a].max() + 1) * B - 1
-        m = max(abs(T0 - S1), abs(T1 - S0))
-        N.append(fft_length(max(2 * m + 2, 2 * (S1 - S0 + 1))))
-    return {"Es": Es, "Et": Et, "N": N, "ncomp": ncomp, "nsrc": len(s), "ndst": len(t)}
+    return {"Es": Es, "Et": Et, "N": list(lengths), "ncomp": ncomp, "nsrc": len(s), "ndst": len(t)}
 
 
 def pass_flops(plan_geom):
@@ -303,13 +298,13 @@ def bench_gpu(args):
     from paper_1601_00035_gb300 import lgf
 
     f, src_c, dst_c, cfg = workload()
-    geom = geometry(src_c, dst_c, 3)
     K = lgf.required_max_offset(src_c, dst_c, B)
     table = lgf.Table(lgf.LAPLACE7, max_offset=K)
-    # the library runs the three components on three streams (one launch per pass
-    # and component); the launch sequence is captured in a CUDA graph on first use
+    # the library runs the three components in each launch of its three passes (or, five passes, on
+    # three streams); the launch sequence is captured in a CUDA graph on first use
     plan = lgf.Plan(table, [lgf.Solve(B, 3, src_c, dst_c, scale=-1.0)], use_graph=True, method=lgf.METHOD_AUTOTUNE)
     chosen, auto_wb, auto_split = plan.method()
+    passes, lengths = plan.lengths()
     stream = torch.cuda.current_stream()
     d_src = torch.from_numpy(f).cuda()
     d_dst = torch.zeros((len(dst_c), 3, B, B, B), device="cuda")
@@ -390,17 +385,17 @@ def bench_gpu(args):
     # roofline of the dominant kernel, on the algorithmic bytes of the path: 8 B per target
     # point (4 B FP32 source in, 4 B result out); one launch of a pass is all three components
     # in the three-pass form, one component in the five-pass form
-    per = 3 if "yz_conv" in kt else 1
-    g1 = geometry(src_c, dst_c, per)
-    pb = pass_bytes(g1)
-    pf = pass_flops(g1)
+    per = 3 if passes == 3 else 1
+    g1 = geometry(src_c, dst_c, per, lengths)
+    # (the autotuner may have chosen the split solve: no per-pass workspace or flop model)
+    pb, pf = (pass_bytes(g1), pass_flops(g1)) if passes else ({}, {})
     dom = max(kt, key=lambda k: kt[k][1])
     launches, tot_ms = kt[dom]
     per_launch_ms = tot_ms / launches
     hbm, src_kind = peaks()
     alg_bytes = 8 * per * len(dst_c) * B ** 3
     achieved = alg_bytes / (per_launch_ms / 1e3) / 1e9
-    if dom not in pb:      # the autotuner chose the split solve: no per-pass workspace or flop model
+    if dom not in pb:
         pb[dom], pf[dom] = 0, 0.0
     step_gbs = 8 * pts_per_step / (dev_ms / args.steps / 1e3) / 1e9
     roof = {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
@@ -415,7 +410,7 @@ def bench_gpu(args):
                                "frac": round(pb[dom] / (per_launch_ms / 1e3) / 1e9 / hbm, 4),
                                "rule": "the pass's own input and output arrays (complex FP32 workspaces, "
                                        "kernel spectrum): bytes of this algorithm, not of the path"},
-            "traffic_note": "DRAM bytes per launch (ncu) are in profiles/poisson_ring128_ncu.md",
+            "traffic_note": "DRAM bytes per launch are counted by ncu, not in this run",
             "launch_timing": "CUDA events around each launch (one pass) in K profiled steps after the timed ones",
             "peak_source": src_kind + " (MEASURED_PEAKS.json hbm_gbs)" if src_kind == "measured" else src_kind}
     comp_tf = pf[dom] / (per_launch_ms / 1e3) / 1e12
@@ -443,7 +438,7 @@ def bench_gpu(args):
     cfg.update({"method": {"chosen": ["whole-box FFT convolution", "block-sparse split solve"][chosen],
                            "autotune_ms": {"whole_box": round(auto_wb, 4), "split": round(auto_split, 4)},
                            "rule": "lgf_conv_plan method 2: both planned, one timed execution each, the faster kept"},
-                "fft_grid": geom["N"], "execution": "%s, launch sequence replayed as a CUDA graph" %
+                "fft_grid": lengths, "execution": "%s, launch sequence replayed as a CUDA graph" %
                 ("three passes, all components per launch" if per == 3 else "one stream per component"),
                 "plain_ms": round(plain_ms, 4), "batched_over_plain": round(plain_ms / (dev_ms / args.steps), 3),
                 "plain": "one component per solve, three solves one after another on one stream, no graph",

@@ -167,6 +167,10 @@ lgf_status lgf_conv_plan(const lgf_table *t, const lgf_solve_desc *solves, int n
  * of the two candidates measured at plan time (-1 where not timed); either pointer may be NULL. */
 int lgf_plan_method(const lgf_plan *p, double *ms_whole_box, double *ms_split);
 
+/* The padded FFT lengths n (x, y, z) on which solve `solve` of a whole-box plan runs, and as return
+ * value its passes: 3 or 5.  0 (n zero) for a split plan, -1 for a bad argument. */
+int lgf_plan_lengths(const lgf_plan *p, int solve, int n[3]);
+
 /* The near-field form that a split plan executes: 1 pairs, 2 runs, 3 quads, 4 quads in
  * shared-memory tiles (opts->near_form = 3 takes 3 or 4); 0 for a whole-box plan, -1 for NULL.
  * ms (may be NULL): ms[i] receives the time of form i + 1 measured at plan time (-1 where not timed). */

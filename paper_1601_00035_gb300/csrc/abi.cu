@@ -1040,6 +1040,19 @@ int lgf_plan_method(const lgf_plan *p, double *ms_whole_box, double *ms_split)
     return p->method;
 }
 
+int lgf_plan_lengths(const lgf_plan *p, int solve, int n[3])
+{
+    if (!p || !n) return -1;
+    if (p->sub) return lgf_plan_lengths(p->sub, solve, n);
+    n[0] = n[1] = n[2] = 0;
+    if (p->split) return 0;
+    if (p->kind != LGF_KERNEL_LAPLACE7 || solve < 0 || solve >= (int)p->solves.size()) return -1;
+    const PoissonSolve &q = p->solves[solve];
+    const int three[3] = {2 * q.pg.Mx, q.pg.Dy * q.pg.My, 2 * q.pg.Mz};
+    for (int a = 0; a < 3; a++) n[a] = q.plane ? three[a] : q.g.N[a];
+    return q.plane ? 3 : 5;
+}
+
 int lgf_plan_near_form(const lgf_plan *p, double ms[4])
 {
     if (!p) return -1;

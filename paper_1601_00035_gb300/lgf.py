@@ -88,6 +88,7 @@ _SIGS = {
     "lgf_plan_workspace_bytes": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_size_t)]),
     "lgf_plan_method": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_double),
                                        ctypes.POINTER(ctypes.c_double)]),
+    "lgf_plan_lengths": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
     "lgf_plan_near_form": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_double)]),
     "lgf_plan_check": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     "lgf_wait_probe": (ctypes.c_int, [ctypes.c_int, ctypes.c_void_p]),
@@ -256,6 +257,11 @@ class Plan:
         a, b = ctypes.c_double(), ctypes.c_double()
         m = load().lgf_plan_method(self._h, ctypes.byref(a), ctypes.byref(b))
         return m, a.value, b.value
+
+    def lengths(self, solve: int = 0):
+        """(passes of a whole-box solve: 3 or 5, its padded FFT lengths [x, y, z]); (0, zeros) for a split plan."""
+        n = (ctypes.c_int * 3)()
+        return load().lgf_plan_lengths(self._h, int(solve), n), list(n)
 
     def near_form(self):
         """(near-field form of a split plan: 1 pairs, 2 runs, 3 quads, 4 quads in tiles; 0 whole box,
