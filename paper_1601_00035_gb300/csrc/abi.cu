@@ -698,7 +698,7 @@ static lgf_status plan_poisson(lgf_plan *p, const lgf_table *t, const lgf_solve_
         p->wsB = maxB;
         if (p->solves[0].g.ncomp == 1) return LGF_OK;
     }
-    // Several independent units, one per (solve, component): each runs the five
+    // Several independent units, one per (solve, component): each runs its
     // passes on its own worker stream (up to 4), so the passes of different
     // units overlap (a memory-bound pass beside the compute-bound z pass).
     // Longest-first greedy assignment, the workspace size as the cost estimate.
@@ -1104,7 +1104,7 @@ static lgf_status run_poisson(lgf_plan *p, const float *const *src, float *const
         g.nc = u.nc;
         return g;
     };
-    // one unit on stream st: host copy in, five passes, host copy out
+    // one unit on stream st: host copy in, three or five passes, host copy out
     // wait (optional): the unit (its copy in included) starts after that event
     auto run_unit = [&](const lgf_plan::Unit &u, cx<float> *wa, cx<float> *wb, cudaStream_t st, Profiler *pr,
                         cudaEvent_t wait = nullptr, cudaEvent_t mark = nullptr) -> lgf_status {
@@ -1123,6 +1123,7 @@ static lgf_status run_poisson(lgf_plan *p, const float *const *src, float *const
         return LGF_OK;
     };
     if (p->grouped) {
+        static_assert(kPlaneMaxSolves >= kGroupMaxSolves, "a grouped plan's buffers fit both kernel parameters");
         SolvePtrs<float> ptrs;
         PlanePtrs pptrs;
         for (size_t i = 0; i < p->solves.size(); i++) {
@@ -1131,7 +1132,7 @@ static lgf_status run_poisson(lgf_plan *p, const float *const *src, float *const
         }
         static const char *pnames[3] = {"x_fwd_gather_r2c", "yz_conv", "x_inv_c2r_scatter"};
         static const char *names[5] = {"x_fwd_gather_r2c", "y_fwd", "z_fwd_mul_inv", "y_inv", "x_inv_c2r_scatter"};
-        // one group on stream st: its units' copies in, five grouped launches, copies out
+        // one group on stream st: its units' copies in, a grouped launch per pass, copies out
         auto run_group = [&](const lgf_plan::Group &gr, cudaStream_t st, Profiler *pr) -> lgf_status {
             if (host)
                 for (int i : gr.units) {

@@ -324,7 +324,7 @@ struct lgf_plan {
     std::vector<Unit> units;
     std::vector<cudaEvent_t> unit_mark;  // per unit: recorded after one of its passes (staggered start)
     // grouped execution (many units): the units with the same FFT grid form a group
-    // whose five passes are five launches over device task tables; the groups run on
+    // whose passes are one launch each over device task tables; the groups run on
     // the worker streams (lanes); every unit has its own workspaces
     bool grouped = false;
     std::vector<lgf::cx<float> *> unit_wa, unit_wb;

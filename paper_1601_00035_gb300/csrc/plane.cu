@@ -248,9 +248,9 @@ lgf_status plane_pass(int pass, const PlaneGeom &g, const float *src, float *dst
 lgf_status plane_pass_grouped(int pass, int M, size_t smem, int threads, int Dy, const PlaneTask *t, const int *cta, int n,
                               const PlanePtrs &p, cudaStream_t s)
 {
-#define LGF_F(L) case L: return PlaneX<L>::fwd_grp(t, cta, n, smem, p, s);
+#define LGF_F(L) case L: return PlaneX<L>::fwd_grp(t, cta, n, p, s);
 #define LGF_Z(L) case L: return PlaneYZ<L>::grp(t, cta, n, smem, threads, Dy, s);
-#define LGF_I(L) case L: return PlaneX<L>::inv_grp(t, cta, n, smem, p, s);
+#define LGF_I(L) case L: return PlaneX<L>::inv_grp(t, cta, n, p, s);
     if (pass == 0) LGF_PLANE_SWITCH(M, LGF_F)
     if (pass == 1) LGF_PLANE_SWITCH(M, LGF_Z)
     LGF_PLANE_SWITCH(M, LGF_I)

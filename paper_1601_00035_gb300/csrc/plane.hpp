@@ -46,8 +46,8 @@ struct PlaneX {
     static lgf_status prepare();
     static lgf_status fwd(const PlaneGeom &g, const float *src, cx<float> *a, cudaStream_t s);
     static lgf_status inv(const PlaneGeom &g, const cx<float> *b, float *dst, cudaStream_t s);
-    static lgf_status fwd_grp(const PlaneTask *t, const int *cta, int ncta, size_t smem, const PlanePtrs &p, cudaStream_t s);
-    static lgf_status inv_grp(const PlaneTask *t, const int *cta, int ncta, size_t smem, const PlanePtrs &p, cudaStream_t s);
+    static lgf_status fwd_grp(const PlaneTask *t, const int *cta, int ncta, const PlanePtrs &p, cudaStream_t s);
+    static lgf_status inv_grp(const PlaneTask *t, const int *cta, int ncta, const PlanePtrs &p, cudaStream_t s);
 };
 template <int M>
 struct PlaneYZ {

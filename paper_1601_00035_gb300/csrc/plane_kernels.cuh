@@ -839,13 +839,13 @@ lgf_status PlaneX<M>::inv(const PlaneGeom &g, const cx<float> *b, float *dst, cu
     return LGF_OK;
 }
 template <int M>
-lgf_status PlaneX<M>::fwd_grp(const PlaneTask *t, const int *cta, int ncta, size_t, const PlanePtrs &p, cudaStream_t s)
+lgf_status PlaneX<M>::fwd_grp(const PlaneTask *t, const int *cta, int ncta, const PlanePtrs &p, cudaStream_t s)
 {
     LGF_CUDA_TRY(launch_pdl_smem(k_px_fwd_grp<M>, dim3(ncta), dim3(PX_THREADS), px_smem<M>(), s, t, cta, p));
     return LGF_OK;
 }
 template <int M>
-lgf_status PlaneX<M>::inv_grp(const PlaneTask *t, const int *cta, int ncta, size_t, const PlanePtrs &p, cudaStream_t s)
+lgf_status PlaneX<M>::inv_grp(const PlaneTask *t, const int *cta, int ncta, const PlanePtrs &p, cudaStream_t s)
 {
     LGF_CUDA_TRY(launch_pdl_smem(k_px_inv_grp<M>, dim3(ncta), dim3(PX_THREADS), px_smem<M>(), s, t, cta, p));
     return LGF_OK;
