@@ -729,7 +729,8 @@ __device__ __forceinline__ void yz_body(const PlaneGeom &g, const C *__restrict_
             C *colp = plane + col * P;
             float kv[R2];
             // the first middle butterfly's spectrum, in flight during the first stage
-            if (plane_mid_any(MZ, b)) z_spectrum<MZ>(kv, Kp, col, My, b >= R1, b >= R1 ? b - R1 : b);
+            const int ahead = plane_mid_ahead(MZ, b);
+            z_spectrum<MZ>(kv, Kp, col, My, ahead >= R1, ahead >= R1 ? ahead - R1 : ahead);
             {
                 V x[R1], v[R1];
 #pragma unroll

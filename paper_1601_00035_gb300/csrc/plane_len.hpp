@@ -29,10 +29,12 @@ LGF_LEN int plane_yz_threads(int M) { return M <= 128 ? 1024 : M <= 192 ? 768 : 
 // The middle of the z convolution.  A column has 2 R1 butterflies of R2 points, u < R1 those of the
 // even frequencies (q = u) and the rest those of the odd ones (q = u - R1); its R2 threads take
 // butterfly b, then b + R2 and so on.  Threads b >= 2 R1 (lengths 96 and 112, where R1 is 6 and 7
-// and R2 is 16) have none.
-LGF_LEN bool plane_mid_any(int M, int b)
+// and R2 is 16) have none: the spectrum that every thread loads ahead is then the last butterfly's,
+// and is dropped (64 ragged solves 1361 us; with a branch around the load 1369).
+LGF_LEN int plane_mid_ahead(int M, int b)
 {
-    return 2 * (M / plane_z2(M)) >= plane_z2(M) || b < 2 * (M / plane_z2(M));  // (the first folds at compile time)
+    const int last = 2 * (M / plane_z2(M)) - 1;
+    return last >= plane_z2(M) - 1 || b < last ? b : last;  // (the first folds at compile time)
 }
 // Spectrum row (0 .. M, plane.cu's order: even frequencies, then odd ones) of element k2 of butterfly
 // q: frequency kk = q + R1 k2 of its half is row plane_row_lo + R1 k2 below M / 2 (k2 < R2 / 2), and

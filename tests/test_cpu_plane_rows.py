@@ -14,33 +14,33 @@ PROGRAM = r"""
 #include <cstdio>
 #include "plane_len.hpp"
 using namespace lgf;
+int bad = 0;
+void load(int M, int b, int u)  // thread b loads the spectrum of butterfly u
+{
+    const int R2 = plane_z2(M), R1 = M / R2;
+    const bool odd = u >= R1;
+    const int q = odd ? u - R1 : u;
+    for (int k2 = 0; k2 < R2; k2++) {
+        const int row = k2 < R2 / 2 ? plane_row_lo(M, odd, q) + k2 * R1 : plane_row_hi(M, odd, q) - k2 * R1;
+        const int kz = 2 * (q + R1 * k2) + odd, f = kz <= M ? kz : 2 * M - kz;
+        const int want = odd ? M / 2 + 1 + f / 2 : f / 2;
+        if (row >= 0 && row <= M && row == want) continue;
+        if (!bad++) printf("length %d, thread %d, k2 %d: row %d of %d, frequency in %d\n", M, b, k2, row, M + 1, want);
+    }
+}
+void length(int M)
+{
+    const int R2 = plane_z2(M), R1 = M / R2;
+    for (int b = 0; b < R2; b++) {
+        const int ahead = plane_mid_ahead(M, b);
+        load(M, b, ahead);
+        if (b < 2 * R1 && ahead != b) bad++, printf("length %d: thread %d loads butterfly %d ahead\n", M, b, ahead);
+        for (int u = b + R2; u < 2 * R1; u += R2) load(M, b, u);
+    }
+}
 int main()
 {
-    int bad = 0;
-#define CHECK(M)                                                                                        \
-    {                                                                                                   \
-        const int R2 = plane_z2(M), R1 = M / R2;                                                        \
-        int seen[2 * 256] = {};                                                                         \
-        for (int b = 0; b < R2; b++)                                                                    \
-            for (int u = b; u == b ? plane_mid_any(M, b) : u < 2 * R1; u += R2) {                       \
-                const bool odd = u >= R1;                                                               \
-                const int q = odd ? u - R1 : u;                                                         \
-                if (u < 2 * R1) seen[u]++;                                                              \
-                for (int k2 = 0; k2 < R2; k2++) {                                                       \
-                    const int row = k2 < R2 / 2 ? plane_row_lo(M, odd, q) + k2 * R1                     \
-                                                : plane_row_hi(M, odd, q) - k2 * R1;                    \
-                    const int kz = 2 * (q + R1 * k2) + odd, f = kz <= M ? kz : 2 * M - kz;              \
-                    const int want = odd ? M / 2 + 1 + f / 2 : f / 2;                                   \
-                    if (row < 0 || row > M || row != want) {                                            \
-                        if (!bad) printf("length %d, thread %d, k2 %d: row %d of %d, frequency in %d\n", \
-                                         M, b, k2, row, M + 1, want);                                   \
-                        bad++;                                                                          \
-                    }                                                                                   \
-                }                                                                                       \
-            }                                                                                           \
-        for (int u = 0; u < 2 * R1; u++)                                                                \
-            if (seen[u] != 1) bad++, printf("length %d: butterfly %d done %d times\n", M, u, seen[u]);  \
-    }
+#define CHECK(M) length(M);
     LGF_PLANE_LENGTHS(CHECK)
     return bad != 0;
 }
